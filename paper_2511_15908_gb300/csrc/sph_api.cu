@@ -234,6 +234,10 @@ sph_status finalize(sph_handle *h)
     c.n = n;
     c.nb = (int)h->bodies.size();
     c.n_body_particles = n - c.nf;
+    c.n_rigid = 0;
+    for (const DevBody &B : h->bodies)
+        if (B.kind == SPH_BODY_RIGID) c.n_rigid += B.n;
+    c.coop = walk_coop(c);
     c.n_force_blocks = (n + 255) / 256;
     if ((h->p.flags & SPH_FLAG_LOW_LATENCY) && !(h->p.flags & SPH_FLAG_VOLUME_BOUNDARY))
         c.n_force_blocks = (int)(((long long)n * kLowLatencyForceG + 255) / 256);

@@ -19,7 +19,7 @@
 
 namespace sphgb {
 
-enum Phase { P_HASH, P_SCAN_T, P_SCAN_A, P_SCATTER, P_GATHER, P_VOLUME, P_DENSITY, P_FORCE, P_WRENCH,
+enum Phase { P_HASH, P_SCAN_T, P_SCAN_A, P_SCATTER, P_GATHER, P_SEARCH, P_VOLUME, P_DENSITY, P_FORCE, P_WRENCH,
              kPhases };
 
 constexpr unsigned kBarrierSpin = 1u << 22;   // x 64 ns sleep: the barrier gives up after ~0.3 s
@@ -126,8 +126,12 @@ __global__ void __launch_bounds__(kTile, SPH_BATCH_MINB) k_batch(BatchConst b, i
                     case P_SCAN_A: scan_apply_item(c, blk); break;
                     case P_SCATTER: scatter_item(c, blk); break;
                     case P_GATHER: rank_gather_item(c, blk); break;
+                    case P_SEARCH: search_item<kTile, 0>(c, blk); break;
                     case P_VOLUME: boundary_volume_item(c, blk); break;
-                    case P_DENSITY: density_item<kTile, false>(c, blk); break;
+                    case P_DENSITY:
+        if (c.flags & FLAG_VOLUME) density_item<kTile, 0, DENSITY_VOLUME, false>(c, blk);
+        else density_item<kTile, 0, DENSITY_MASS, false>(c, blk);
+        break;
                     case P_FORCE: force_item(c, blk); break;
                     default: wrench_item(c, blk); break;
                     }
@@ -146,11 +150,11 @@ __global__ void __launch_bounds__(kTile, SPH_BATCH_MINB) k_batch(BatchConst b, i
 
 // Per-phase alternative: one kernel per phase whose blocks are that phase's tiles over all
 // scenes (no grid barrier; each phase keeps its own register budget and occupancy).
-// Resident blocks per SM each phase is built for.  Without a bound the density phase took
-// 64 registers (4 blocks); 5 blocks give 51 without spilling (6 spill: the scene's
-// parameters live in shared memory here), per-phase batch 4.29 -> 3.90 ms on 64 scenes.
+// Resident blocks per SM each phase is built for (64 scenes of 0.5k-2k fluid, 356k particles:
+// density at 5 blocks 441 us a substep against 428 at 4, 435 at 3; the search at 4 and 5 the
+// same).
 template <int PH>
-constexpr int batch_phase_minb() { return PH == P_DENSITY ? 4 : PH == P_FORCE ? 3 : 1; }
+constexpr int batch_phase_minb() { return PH == P_SEARCH ? 5 : PH == P_DENSITY ? 4 : PH == P_FORCE ? 3 : 1; }
 
 template <int PH>
 __global__ void __launch_bounds__(kTile, batch_phase_minb<PH>()) k_batch_phase(BatchConst b)
@@ -173,8 +177,12 @@ __global__ void __launch_bounds__(kTile, batch_phase_minb<PH>()) k_batch_phase(B
     case P_SCAN_A: scan_apply_item(c, blk); break;
     case P_SCATTER: scatter_item(c, blk); break;
     case P_GATHER: rank_gather_item(c, blk); break;
+    case P_SEARCH: search_item<kTile, 0>(c, blk); break;
     case P_VOLUME: boundary_volume_item(c, blk); break;
-    case P_DENSITY: density_item<kTile, false>(c, blk); break;
+    case P_DENSITY:
+        if (c.flags & FLAG_VOLUME) density_item<kTile, 0, DENSITY_VOLUME, false>(c, blk);
+        else density_item<kTile, 0, DENSITY_MASS, false>(c, blk);
+        break;
     case P_FORCE: force_item(c, blk); break;
     default: wrench_item(c, blk); break;
     }
@@ -264,6 +272,7 @@ cudaError_t launch_phases(sph_batch *b, int n_substeps, int cycle_end)
         if (bc.total[P_SCAN_A]) k_batch_phase<P_SCAN_A><<<bc.total[P_SCAN_A], kTile, 0, b->stream>>>(bc);
         if (bc.total[P_SCATTER]) k_batch_phase<P_SCATTER><<<bc.total[P_SCATTER], kTile, 0, b->stream>>>(bc);
         if (bc.total[P_GATHER]) k_batch_phase<P_GATHER><<<bc.total[P_GATHER], kTile, 0, b->stream>>>(bc);
+        if (bc.total[P_SEARCH]) k_batch_phase<P_SEARCH><<<bc.total[P_SEARCH], kTile, 0, b->stream>>>(bc);
         if (bc.total[P_VOLUME]) k_batch_phase<P_VOLUME><<<bc.total[P_VOLUME], kTile, 0, b->stream>>>(bc);
         if (bc.total[P_DENSITY]) k_batch_phase<P_DENSITY><<<bc.total[P_DENSITY], kTile, 0, b->stream>>>(bc);
         if (bc.total[P_FORCE]) k_batch_phase<P_FORCE><<<bc.total[P_FORCE], kTile, 0, b->stream>>>(bc);
@@ -406,6 +415,7 @@ sph_status sph_batch_create(sph_handle *const *scenes, int32_t n_scenes, void *d
         // them give the same results (a batch fills the GPU; the low-latency pass is not
         // what it needs)
         table[s].flags &= ~FLAG_LOW_LATENCY;
+        table[s].coop = 0;
         table[s].n_force_blocks = (table[s].n + 255) / 256;
     }
     sph_batch *b = new sph_batch();
@@ -427,7 +437,9 @@ sph_status sph_batch_create(sph_handle *const *scenes, int32_t n_scenes, void *d
             const SimConst &c = table[s];
             int tiles = (ph == P_SCAN_T || ph == P_SCAN_A) ? c.n_scan_tiles
                         : (ph == P_WRENCH) ? c.n_wgrid
-                        : (ph == P_VOLUME && !(c.flags & FLAG_VOLUME)) ? 0
+                        : (ph == P_VOLUME) ? ((c.flags & FLAG_VOLUME) ? (c.n - c.nf + kTile - 1) / kTile : 0)
+                        : (ph == P_SEARCH) ? search_tiles(c, kTile)
+                        : (ph == P_DENSITY) ? density_tiles(c, kTile)
                         : (c.n + kTile - 1) / kTile;
             run += tiles;
         }

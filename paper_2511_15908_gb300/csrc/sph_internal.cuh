@@ -49,6 +49,9 @@ struct DevBody {
 // Everything a substep kernel needs, passed by value (lives in the constant bank).
 struct __align__(16) SimConst {
     int n, nf, nb, n_body_particles;
+    int n_rigid;               // particles of rigid bodies
+    int coop;                  // who walks with cooperating lanes (walk_role): 0 nobody, 1 rigid
+                               // particles, 2 every particle
     int nx, ny, nz, ncell;
     float o[3], inv_cell;
     float R2, h, inv_h;
@@ -81,7 +84,7 @@ struct __align__(16) SimConst {
     unsigned long long *tile_state;   // n_scan_tiles + 1 words of the single-pass scan: per
                                       // tile (kind << 32 | value), then the tile counter;
                                       // zeroed by the hash pass before every scan
-    int *slot_of_id;           // id -> sorted slot (soft particles only)
+    int *slot_of_id;           // id -> sorted slot (body particles)
     float4 *locals;            // per body particle (id - nf): body-frame offset
     int *spring_row;           // per body particle (id - nf), CSR row start (+1 entry)
     float4 *spring_e;          // (partner id bits, L0, k_s, c_d)
@@ -115,6 +118,8 @@ constexpr int kSubstepKernels = 8;
 cudaError_t launch_substep(const SimConst &c, cudaStream_t s, cudaEvent_t *ev = nullptr,
                            bool external = false, bool cycle_end = false,
                            unsigned ev_mask = ~0u);
+// who walks with cooperating lanes in a scene stepped alone
+int walk_coop(const SimConst &c);
 // the events around the density pass alone (events 5 and 6)
 constexpr unsigned kDensityEvents = (1u << 5) | (1u << 6);
 // spring cutting against a blade triangle (sorts the current state first, like the next

@@ -3,22 +3,15 @@
 #include "sph_device.cuh"
 
 // Block shape and resident blocks per SM each pass is built for (its register budget).
-// Measured on the 1.16 M-particle coupled scene: density in 512-thread blocks, 2 per SM (62
-// registers) 305 us, against 317 for 256 x 4, 354 for 256 x 6 (40 registers), 320 for
-// 128 x 8 and 316 for 1024 x 1; force in 256-thread blocks, 5 per SM, with two neighbours'
-// loads in flight 136 us against 146 at 4 and 158 at 6.  Scenes too small to fill two
-// waves of the wide blocks (kDensityWideMin particles) take 256 x 4: on 64 scenes of
-// 8k-256k particles the wide blocks alone cost 4 % more.
-#ifndef SPH_DENSITY_THREADS
-#define SPH_DENSITY_THREADS 512
-#endif
-#ifndef SPH_DENSITY_MINB
-#define SPH_DENSITY_MINB 2
-#endif
+// Measured (us, search + sums): search in 256-thread blocks at 5 blocks per SM, 48 registers
+// (6 blocks, 40 registers: coupled 1.16 M 437 against 409; 4: the same); density sums at 4
+// blocks, 64 registers, with the next quad's neighbours in flight (5 blocks spill: 476 against
+// 414; 3 blocks: 422); force in 256-thread blocks with two neighbours' loads in flight.
+#define SPH_DENSITY_THREADS 256
+#define SPH_DENSITY_MINB 4
 #ifndef SPH_FORCE_MINB
 #define SPH_FORCE_MINB 4
 #endif
-constexpr int kDensityWideMin = 300000;   // ~ 2 x 152 SMs x 2 blocks x 512 threads
 // Low-latency density pass (SPH_FLAG_LOW_LATENCY): G lanes per particle, 32 up to
 // kLowLatency32Max particles, else 16.  Measured (density pass, us) on the dam break (12k
 // particles) / a compact stirring tank (4.8k) / the coupled scene with 60k fluid (83k):
@@ -42,23 +35,23 @@ __global__ void __launch_bounds__(kTile) k_scan_lookback(SimConst c) { scan_look
 #endif
 __global__ void __launch_bounds__(kTile) k_scatter(SimConst c) { scatter_item(c, blockIdx.x); }
 __global__ void __launch_bounds__(kTile) k_rank_gather(SimConst c) { rank_gather_item(c, blockIdx.x); }
+template <int COOP, int MODE>
 __global__ void __launch_bounds__(SPH_DENSITY_THREADS, SPH_DENSITY_MINB) k_density(SimConst c)
 {
-    density_item<SPH_DENSITY_THREADS>(c, blockIdx.x);
+    density_item<SPH_DENSITY_THREADS, COOP, MODE, true>(c, blockIdx.x);
 }
-__global__ void __launch_bounds__(kTile, 4) k_density_narrow(SimConst c) { density_item<kTile>(c, blockIdx.x); }
+#define SPH_SEARCH_THREADS 256
+#define SPH_SEARCH_MINB 5
+template <int COOP>
+__global__ void __launch_bounds__(SPH_SEARCH_THREADS, SPH_SEARCH_MINB) k_search(SimConst c)
+{
+    search_item<SPH_SEARCH_THREADS, COOP>(c, blockIdx.x);
+}
 template <int G>
 __global__ void __launch_bounds__(kTile, SPH_LOW_LATENCY_MINB) k_density_coop(SimConst c)
 {
     density_coop_item<G>(c, blockIdx.x);
 }
-#if SPH_DENSITY_BRICK
-__global__ void __launch_bounds__(kBrickThreads, 2) k_density_brick(SimConst c)
-{
-    extern __shared__ __align__(16) unsigned char dsm[];
-    density_brick(c, *reinterpret_cast<BrickShared *>(dsm));
-}
-#endif
 __global__ void __launch_bounds__(kTile) k_boundary_volume(SimConst c) { boundary_volume_item(c, blockIdx.x); }
 __global__ void __launch_bounds__(kTile, SPH_FORCE_MINB) k_force(SimConst c) { force_item(c, blockIdx.x); }
 template <int G>
@@ -113,6 +106,24 @@ __global__ void k_sorted_keys(SimConst c, uint32_t *keys, int *ids)
 
 // ----------------------------------------------------------------------- launchers
 
+// Who walks with cooperating lanes (same results either way; us of search + density sum):
+//   every particle, 16 lanes, in scenes of up to 60,000: dam break (12k particles) 31 (8 lanes
+//     41, 32 lanes 38) against 112 with one thread each, where a cube particle's ~226
+//     neighbours form one chain; 45k particles of the coupled scene 71.6 against 75; a 58k
+//     stirring tank 127 against 137; 85k of the coupled scene 113 against 78;
+//   rigid particles, 4 lanes, up to 900,000 particles: 307k of the coupled scene 103 against
+//     159, the 365k stirring tank (18.7k of them rigid) 156 against 184; 2 lanes 161 / 160,
+//     8 lanes 108 / 166.  The 1.16 M coupled scene lasts longer than its rigid chains (389 with
+//     4 lanes against 385).  With more than an eighth of all particles rigid their number hides
+//     the chains, and the lanes' overhead would show;
+//   nobody else.
+constexpr int kCoopAllMax = 60000, kCoopRigidMax = 900000;
+int walk_coop(const SimConst &c)
+{
+    if (c.Rc >= 2.5f) return 0;                 // the cooperative search's row table
+    return c.n <= kCoopAllMax ? 2 : c.n <= kCoopRigidMax && c.n_rigid <= c.n / 8 ? 1 : 0;
+}
+
 static inline int blocks_for(int n, int t) { return (n + t - 1) / t; }
 
 cudaError_t launch_substep(const SimConst &c, cudaStream_t s, cudaEvent_t *ev, bool external,
@@ -140,29 +151,23 @@ cudaError_t launch_substep(const SimConst &c, cudaStream_t s, cudaEvent_t *ev, b
     mark();
     k_rank_gather<<<nb, kTile, 0, s>>>(c);
     mark();
-    // volume-based boundaries: their weights first (timed with the density pass)
-    if (c.flags & FLAG_VOLUME) k_boundary_volume<<<nb, kTile, 0, s>>>(c);
-#if SPH_DENSITY_BRICK
-    static bool brick_attr = false;
-    if (!brick_attr) {
-        cudaFuncSetAttribute(k_density_brick, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(BrickShared));
-        brick_attr = true;
+    // the neighbour search and the sums over its lists (timed together); the volume variant's
+    // boundary weights between them.  The low-latency pass searches for itself; its group's
+    // rows fit its 6 x 6 table while Rc < 2.5 (cells >= h give Rc ~ 2)
+    if ((c.flags & FLAG_LOW_LATENCY) && !(c.flags & FLAG_VOLUME) && c.Rc < 2.5f) {
+        if (c.n <= kLowLatency32Max)
+            k_density_coop<32><<<(unsigned)(((long long)c.n * 32 + kTile - 1) / kTile), kTile, 0, s>>>(c);
+        else
+            k_density_coop<16><<<(unsigned)(((long long)c.n * 16 + kTile - 1) / kTile), kTile, 0, s>>>(c);
+    } else {
+        const auto search = c.coop == 0 ? k_search<0> : c.coop == 1 ? k_search<1> : k_search<2>;
+        search<<<search_tiles(c, SPH_SEARCH_THREADS), SPH_SEARCH_THREADS, 0, s>>>(c);
+        const bool vol = (c.flags & FLAG_VOLUME) != 0;
+        if (vol && c.n > c.nf) k_boundary_volume<<<blocks_for(c.n - c.nf, kTile), kTile, 0, s>>>(c);
+        const auto density = vol ? (c.coop == 0 ? k_density<0, DENSITY_VOLUME> : c.coop == 1 ? k_density<1, DENSITY_VOLUME> : k_density<2, DENSITY_VOLUME>)
+                                 : (c.coop == 0 ? k_density<0, DENSITY_MASS> : c.coop == 1 ? k_density<1, DENSITY_MASS> : k_density<2, DENSITY_MASS>);
+        density<<<density_tiles(c, SPH_DENSITY_THREADS), SPH_DENSITY_THREADS, 0, s>>>(c);
     }
-    if (c.n >= kDensityWideMin && !(c.flags & FLAG_VOLUME))
-        k_density_brick<<<dim3((c.nx + kBX - 1) / kBX, (c.ny + kBY - 1) / kBY, (c.nz + kBZ - 1) / kBZ), kBrickThreads,
-                          sizeof(BrickShared), s>>>(c);
-    else
-#endif
-    // the group's rows fit its 6 x 6 table while Rc < 2.5 (cells >= h give Rc ~ 2)
-    if ((c.flags & FLAG_LOW_LATENCY) && !(c.flags & FLAG_VOLUME) && c.Rc < 2.5f && c.n <= kLowLatency32Max)
-        k_density_coop<32><<<(unsigned)(((long long)c.n * 32 + kTile - 1) / kTile), kTile, 0, s>>>(c);
-    else if ((c.flags & FLAG_LOW_LATENCY) && !(c.flags & FLAG_VOLUME) && c.Rc < 2.5f)
-        k_density_coop<16><<<(unsigned)(((long long)c.n * 16 + kTile - 1) / kTile), kTile, 0, s>>>(c);
-    else
-    if (c.n >= kDensityWideMin)
-        k_density<<<blocks_for(c.n, SPH_DENSITY_THREADS), SPH_DENSITY_THREADS, 0, s>>>(c);
-    else
-        k_density_narrow<<<nb, kTile, 0, s>>>(c);
     mark();
     // (a flagged scene's n_force_blocks counts blocks of 256 / G particles)
     if ((c.flags & FLAG_LOW_LATENCY) && !(c.flags & FLAG_VOLUME))
