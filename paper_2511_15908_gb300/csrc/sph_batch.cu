@@ -315,9 +315,12 @@ cudaError_t launch_branches(sph_batch *b, int n_substeps, int cycle_end)
         e = cudaEventRecord(b->fork, b->stream);
         for (int k = 0; e == cudaSuccess && k < b->n_branches; ++k)
             e = cudaStreamWaitEvent(b->branch[k], b->fork, 0);
-        for (int sc = 0; e == cudaSuccess && sc < b->n; ++sc)
+        for (int sc = 0; e == cudaSuccess && sc < b->n; ++sc) {
+            SimConst c = b->table[sc];
+            c.n_force_blocks = (c.n + kForceThreads - 1) / kForceThreads;   // launched alone
             for (int i = 0; e == cudaSuccess && i < n_substeps; ++i)
-                e = launch_substep(b->table[sc], b->branch[b->branch_of[sc]]);
+                e = launch_substep(c, b->branch[b->branch_of[sc]]);
+        }
         for (int k = 0; e == cudaSuccess && k < b->n_branches; ++k) {
             e = cudaEventRecord(b->join[k], b->branch[k]);
             if (e == cudaSuccess) e = cudaStreamWaitEvent(b->stream, b->join[k], 0);

@@ -21,6 +21,7 @@ constexpr int kMaxCell = 512;       // particles per cell for the deterministic 
 #define SPH_LOW_LATENCY_FORCE_G 8
 #endif
 constexpr int kLowLatencyForceG = SPH_LOW_LATENCY_FORCE_G;
+constexpr int kForceThreads = 128;  // particles per block (and diagnostic row) of the force pass
 constexpr int kScanTile = 2048;     // cells per scan block (256 threads x 8)
 constexpr int kReduceChunk = 256;   // body particles per wrench-reduction block
 constexpr int kWrenchMinBlocks = 128; // the FP64 reduction is spread over at least this many

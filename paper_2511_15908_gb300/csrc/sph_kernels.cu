@@ -6,12 +6,15 @@
 // Measured (us, search + sums): search in 256-thread blocks at 5 blocks per SM, 48 registers
 // (6 blocks, 40 registers: coupled 1.16 M 437 against 409; 4: the same); density sums at 4
 // blocks, 64 registers, with the next quad's neighbours in flight (5 blocks spill: 476 against
-// 414; 3 blocks: 422); force in 256-thread blocks with two neighbours' loads in flight.
+// 414; 3 blocks: 422); force in 128-thread blocks, 6 per SM, 80 registers: the pass waits for its
+// gathers (4 bytes of list and 40 of state a partner), which more warps hide better than loads
+// issued ahead (coupled 1.16 M: 224; 5 blocks of 96 registers 233, the next two partners
+// fetched ahead at 5 / 4 blocks 297 / 264, 7 blocks 227), and blocks of 256 leave a longer last
+// wave (234 at 3 per SM, 252 at 4 with the spills of 64 registers).
 #define SPH_DENSITY_THREADS 256
 #define SPH_DENSITY_MINB 4
-#ifndef SPH_FORCE_MINB
-#define SPH_FORCE_MINB 4
-#endif
+#define SPH_FORCE_MINB 6
+#define SPH_FORCE_COOP_MINB 3
 // Low-latency density pass (SPH_FLAG_LOW_LATENCY): G lanes per particle, 32 up to
 // kLowLatency32Max particles, else 16.  Measured (density pass, us) on the dam break (12k
 // particles) / a compact stirring tank (4.8k) / the coupled scene with 60k fluid (83k):
@@ -53,9 +56,13 @@ __global__ void __launch_bounds__(kTile, SPH_LOW_LATENCY_MINB) k_density_coop(Si
     density_coop_item<G>(c, blockIdx.x);
 }
 __global__ void __launch_bounds__(kTile) k_boundary_volume(SimConst c) { boundary_volume_item(c, blockIdx.x); }
-__global__ void __launch_bounds__(kTile, SPH_FORCE_MINB) k_force(SimConst c) { force_item(c, blockIdx.x); }
+template <bool VOL>
+__global__ void __launch_bounds__(kForceThreads, SPH_FORCE_MINB) k_force(SimConst c)
+{
+    force_item_v<kForceThreads, VOL>(c, blockIdx.x);
+}
 template <int G>
-__global__ void __launch_bounds__(kTile, SPH_FORCE_MINB) k_force_coop(SimConst c)
+__global__ void __launch_bounds__(kTile, SPH_FORCE_COOP_MINB) k_force_coop(SimConst c)
 {
     force_coop_item<G>(c, blockIdx.x);
 }
@@ -172,8 +179,10 @@ cudaError_t launch_substep(const SimConst &c, cudaStream_t s, cudaEvent_t *ev, b
     // (a flagged scene's n_force_blocks counts blocks of 256 / G particles)
     if ((c.flags & FLAG_LOW_LATENCY) && !(c.flags & FLAG_VOLUME))
         k_force_coop<kLowLatencyForceG><<<c.n_force_blocks, kTile, 0, s>>>(c);
+    else if (c.flags & FLAG_VOLUME)
+        k_force<true><<<c.n_force_blocks, kForceThreads, 0, s>>>(c);
     else
-        k_force<<<c.n_force_blocks, kTile, 0, s>>>(c);
+        k_force<false><<<c.n_force_blocks, kForceThreads, 0, s>>>(c);
     mark();
     if (cycle_end) k_wrench_cycle<<<c.n_wgrid, kTile, 0, s>>>(c);
     else k_wrench<<<c.n_wgrid, kTile, 0, s>>>(c);
