@@ -254,7 +254,7 @@ sph_status finalize(sph_handle *h)
         c.wfirst[b] = (int)wb.size();
         if (!want) continue;
         for (int l0 = 0; l0 < B.n; l0 += kReduceChunk)
-            wb.push_back(make_int4(b, l0, std::min(B.n, l0 + kReduceChunk), 0));
+            wb.push_back(make_int4(b, l0, std::min(B.n, l0 + kReduceChunk), B.first - c.nf));
         c.wcount[b] = (int)wb.size() - c.wfirst[b];
     }
     if ((int)wb.size() > h->L.max_wblocks) return fail(h, SPH_ERR_CAPACITY, "too many reduction blocks");

@@ -96,7 +96,7 @@ struct __align__(16) SimConst {
     float *path;               // max_path x 13
     double *wrench;            // kMaxBodies x 6
     double *wrench_part;       // n_wblocks x 6
-    int4 *wblock;              // (body, l0, l1, 0) per reduction block
+    int4 *wblock;              // (body, l0, l1, first - nf) per reduction block
     double *diag_part;         // n_force_blocks x 8
     double *diag_part2;        // wrench grid x 8 (second level)
     uint4 *nlist4;             // (nl_cap / 4) x n quads: the neighbours the density pass
