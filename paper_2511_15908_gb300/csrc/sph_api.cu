@@ -21,9 +21,13 @@ namespace {
 
 size_t align256(size_t x) { return (x + 255) & ~size_t(255); }
 
+// Up to here (18k particles) the state is read in one copy through pinned memory: three copies
+// to the caller's pageable memory wait for the GPU one by one.
+constexpr size_t kPinStateMax = 512 << 10;
+
 struct Layout {
     size_t xA, vA, xB, vB, prho, key, rank, perm, cnt, cell_start, tile_sum, tile_state, slot_of_id, locals,
-        spring_row, spring_e, fb, xb, acc_dbg, nnbr, body, path, wrench, wrench_part, wblock,
+        spring_row, spring_e, fb, xb, acc_dbg, nnbr, body, path, wrench, wrench_part, wblock, out,
         diag_part, diag_part2, nlist, nlist_n, cut, diag, wlog, cyc_log, status, ctr, total;
     int dims[3], ncell, n_scan_tiles, max_wblocks, max_force_blocks, nl_cap;
 };
@@ -93,6 +97,7 @@ Layout make_layout(const sph_params &p, const sph_capacity &cap)
     L.wrench = take(8 * 6 * kMaxBodies);
     L.wrench_part = take(8 * 6 * (size_t)L.max_wblocks);
     L.wblock = take(16 * (size_t)L.max_wblocks);
+    L.out = take(256 + 44 * N);
     L.diag_part = take(8 * 8 * (size_t)L.max_force_blocks);
     L.diag_part2 = take(8 * 8 * (size_t)std::max(L.max_wblocks, kWrenchMinBlocks));
     L.nl_cap = ((cap.max_neighbours > 0 ? cap.max_neighbours : kDefaultNeighbours) + 3) & ~3;
@@ -138,6 +143,7 @@ struct sph_handle {
     // 64 on): the copies are truly asynchronous and one stream synchronisation ends a read
     unsigned char *pin = nullptr;
     size_t pin_bytes = 0;
+    char *pin_state = nullptr;           // a small scene's state, in the same memory behind them
 };
 
 namespace {
@@ -449,10 +455,15 @@ sph_status sph_create(const sph_params *p, const sph_capacity *cap, void *d_work
     // pinned staging for the synchronising reads: status, then the counters and the
     // smoothing window's cycle log (host memory; unpinned copies if refused)
     h->pin_bytes = 64 + 16 + 48 * (size_t)c.smooth_window;
-    if (cudaHostAlloc((void **)&h->pin, h->pin_bytes, cudaHostAllocDefault) != cudaSuccess) {
+    const size_t pin_end = align256(h->pin_bytes);
+    const size_t state_bytes = 256 + 28 * (size_t)cap->max_particles;
+    const bool small = state_bytes <= kPinStateMax;
+    if (cudaHostAlloc((void **)&h->pin, pin_end + (small ? kPinStateMax : 0), cudaHostAllocDefault) != cudaSuccess) {
         h->pin = nullptr;
         h->pin_bytes = 0;
         cudaGetLastError();
+    } else {
+        if (small) h->pin_state = reinterpret_cast<char *>(h->pin + pin_end);
     }
     *out = h;
     return SPH_OK;
@@ -759,26 +770,52 @@ sph_status sph_get_state(sph_handle *h, float *h_x, float *h_v, float *h_rho, in
     sph_status st = finalize(h);
     if (st != SPH_OK) return st;
     const int n = h->c.n;
-    std::vector<float4> x(n), v(n), acc(h_acc ? n : 0);
-    std::vector<float2> pr(h_rho ? n : 0);
-    std::vector<int> nn(h_nnbr ? n : 0);
+    if (n == 0) return read_status(h);
+    // put in id order on the GPU, then each array goes straight to the caller's memory
+    char *out = at<char>(h, h->L.out);
+    unsigned *d_bad = reinterpret_cast<unsigned *>(out);
+    StateOut o;
+    size_t off = 256;
+    auto place = [&](bool want, size_t bytes) -> char * {
+        char *r = want ? out + off : nullptr;
+        off += want ? bytes * (size_t)n : 0;
+        return r;
+    };
+    o.x = reinterpret_cast<float *>(place(h_x != nullptr, 12));
+    o.v = reinterpret_cast<float *>(place(h_v != nullptr, 12));
+    o.rho = reinterpret_cast<float *>(place(h_rho != nullptr, 4));
+    o.nnbr = reinterpret_cast<int *>(place(h_nnbr != nullptr, 4));
+    o.acc = reinterpret_cast<float *>(place(h_acc != nullptr, 12));
+    o.bad = d_bad;
     cudaStream_t s = h->stream;
-    SPH_CUDA(h, cudaMemcpyAsync(x.data(), h->c.xB, 16 * (size_t)n, cudaMemcpyDeviceToHost, s));
-    SPH_CUDA(h, cudaMemcpyAsync(v.data(), h->c.vB, 16 * (size_t)n, cudaMemcpyDeviceToHost, s));
-    if (h_rho) SPH_CUDA(h, cudaMemcpyAsync(pr.data(), h->c.prho, 8 * (size_t)n, cudaMemcpyDeviceToHost, s));
-    if (h_nnbr) SPH_CUDA(h, cudaMemcpyAsync(nn.data(), h->c.nnbr, 4 * (size_t)n, cudaMemcpyDeviceToHost, s));
-    if (h_acc) SPH_CUDA(h, cudaMemcpyAsync(acc.data(), h->c.acc_dbg, 16 * (size_t)n, cudaMemcpyDeviceToHost, s));
-    st = read_status(h);
-    for (int p = 0; p < n; ++p) {
-        int id;
-        std::memcpy(&id, &v[p].w, 4);
-        if (id < 0 || id >= n) return fail(h, SPH_ERR_STATE, "corrupt particle id");
-        if (h_x) { h_x[3 * id] = x[p].x; h_x[3 * id + 1] = x[p].y; h_x[3 * id + 2] = x[p].z; }
-        if (h_v) { h_v[3 * id] = v[p].x; h_v[3 * id + 1] = v[p].y; h_v[3 * id + 2] = v[p].z; }
-        if (h_rho) h_rho[id] = pr[p].x;
-        if (h_nnbr) h_nnbr[id] = nn[p];
-        if (h_acc) { h_acc[3 * id] = acc[p].x; h_acc[3 * id + 1] = acc[p].y; h_acc[3 * id + 2] = acc[p].z; }
+    SPH_CUDA(h, cudaMemsetAsync(d_bad, 0, 4, s));
+    SPH_CUDA(h, launch_state(h->c, s, o));
+    unsigned bad = 0;
+    if (h->pin_state && off <= kPinStateMax) {
+        // a small scene's arrays and status words in one copy through pinned memory
+        SPH_CUDA(h, cudaMemcpyAsync(h->pin_state, out, off, cudaMemcpyDeviceToHost, s));
+        SPH_CUDA(h, cudaStreamSynchronize(s));
+        auto take = [&](void *dst, const void *d, size_t bytes) {
+            if (dst) std::memcpy(dst, h->pin_state + ((const char *)d - out), bytes * (size_t)n);
+        };
+        take(h_x, o.x, 12);
+        take(h_v, o.v, 12);
+        take(h_rho, o.rho, 4);
+        take(h_nnbr, o.nnbr, 4);
+        take(h_acc, o.acc, 12);
+        uint32_t words[4];
+        std::memcpy(words, h->pin_state, 16);
+        bad = words[0];
+        st = eval_status(h, words + 1);
+    } else {
+        if (h_x) SPH_CUDA(h, cudaMemcpyAsync(h_x, o.x, 12 * (size_t)n, cudaMemcpyDeviceToHost, s));
+        if (h_v) SPH_CUDA(h, cudaMemcpyAsync(h_v, o.v, 12 * (size_t)n, cudaMemcpyDeviceToHost, s));
+        if (h_rho) SPH_CUDA(h, cudaMemcpyAsync(h_rho, o.rho, 4 * (size_t)n, cudaMemcpyDeviceToHost, s));
+        if (h_nnbr) SPH_CUDA(h, cudaMemcpyAsync(h_nnbr, o.nnbr, 4 * (size_t)n, cudaMemcpyDeviceToHost, s));
+        if (h_acc) SPH_CUDA(h, cudaMemcpyAsync(h_acc, o.acc, 12 * (size_t)n, cudaMemcpyDeviceToHost, s));
+        st = read_status_with(h, d_bad, 4, &bad);
     }
+    if (bad) return fail(h, SPH_ERR_STATE, "corrupt particle id");
     return st;
 }
 

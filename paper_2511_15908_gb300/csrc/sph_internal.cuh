@@ -128,6 +128,14 @@ constexpr unsigned kDensityEvents = (1u << 5) | (1u << 6);
 cudaError_t launch_cut(const SimConst &c, cudaStream_t s, const float tri[9], unsigned *count);
 // the first five substep kernels only: hash, scan, reorder of the current state
 cudaError_t launch_sort(const SimConst &c, cudaStream_t s);
+// the state by particle id, what is wanted of it (else null); bad: an id out of range, then the
+// status words
+struct StateOut {
+    float *x, *v, *rho, *acc;  // 3, 3, 1, 3 per particle
+    int *nnbr;
+    unsigned *bad;
+};
+cudaError_t launch_state(const SimConst &c, cudaStream_t s, const StateOut &o);
 cudaError_t launch_cycle_end(const SimConst &c, cudaStream_t s);
 cudaError_t launch_set_grab(const SimConst &c, cudaStream_t s, int body, int grab,
                             const float *pose_vel13, const float *grab_local, int set_pose,
