@@ -60,87 +60,12 @@ __global__ void k_refresh_bf16(const float *master, __nv_bfloat16 *w1, __nv_bflo
     if (t < kOutPad) b4pad[t] = t < kOut ? master[kOffB4 + t] : 0.0f;
 }
 
-// Standardised BF16 input rows xb[b][c] (zero-padded to 272 columns) and, when xbT is given,
-// the column-major copy xbT[c][b]: a 32 x 32 tile per block, transposed through shared memory
-// so that both copies are written along their contiguous dimension.
-__global__ void k_prep_input(const float *x, int B, const float *mean, const float *inv_std,
-                             __nv_bfloat16 *xb, __nv_bfloat16 *xbT, int ldt)
-{
-    __shared__ __nv_bfloat16 tile[32][33];
-    const int c0 = blockIdx.x * 32, b0 = blockIdx.y * 32;
-    const int tx = threadIdx.x, ty = threadIdx.y;
-    for (int r = ty; r < 32; r += blockDim.y) {
-        const int b = b0 + r, c = c0 + tx;
-        if (b < B && c < kInPad) {
-            const float v = c < kIn ? (x[(size_t)b * kIn + c] - mean[c]) * inv_std[c] : 0.0f;
-            const __nv_bfloat16 h = __float2bfloat16_rn(v);
-            xb[(size_t)b * kInPad + c] = h;
-            tile[r][tx] = h;
-        }
-    }
-    if (!xbT) return;
-    __syncthreads();
-    for (int r = ty; r < 32; r += blockDim.y) {
-        const int c = c0 + r, b = b0 + tx;
-        if (b < B && c < kInPad) xbT[(size_t)c * ldt + b] = tile[tx][r];
-    }
-}
-
-__global__ void k_output(const float *y, int B, const float *mean, const float *std_, float *out)
-{
-    const int t = blockIdx.x * blockDim.x + threadIdx.x;
-    if (t >= B * kOut) return;
-    int b = t / kOut, j = t % kOut;
-    out[t] = y[(size_t)b * kOutPad + j] * std_[j] + mean[j];
-}
-
-// MSE on standardised outputs: L = mean over B x 6 of (y - tn)^2; dY = 2 (y - tn) / (6 B),
-// written row-major (the A operand of dZ3 = dY W4) and column-major (the B operand of dW4)
-// in BF16.  One element per thread (16 rows of 16 columns per block); each block writes its
-// FP64 share of the squared error and its FP32 column sums of the unrounded dY (the bias
-// gradient db4), both added in a fixed order here and, block by block, by the gather.
-constexpr int kLossThreads = 256;
-__global__ void k_loss_grad(const float *y, const float *t, int B, const float *mean, const float *inv_std,
-                            __nv_bfloat16 *dyb, __nv_bfloat16 *dybT, int ldt, double *loss_part, float *db4_part)
-{
-    __shared__ double s[kLossThreads];
-    __shared__ float sg[kLossThreads];
-    const int i = blockIdx.x * kLossThreads + threadIdx.x;
-    double acc = 0.0;
-    if (i < B * kOutPad) {
-        const int b = i / kOutPad, j = i % kOutPad;
-        float g = 0.0f;
-        if (j < kOut) {
-            const float tn = (t[(size_t)b * kOut + j] - mean[j]) * inv_std[j];
-            const float d = y[i] - tn;
-            acc = (double)d * d;
-            g = 2.0f * d / (float)(kOut * B);
-        }
-        const __nv_bfloat16 h = __float2bfloat16_rn(g);
-        dyb[i] = h;
-        dybT[(size_t)j * ldt + b] = h;
-        sg[threadIdx.x] = g;
-    } else {
-        sg[threadIdx.x] = 0.0f;
-    }
-    s[threadIdx.x] = acc;
-    __syncthreads();
-    if (threadIdx.x < kOutPad) {               // column j = threadIdx.x of the block's 16 rows
-        float c = 0.0f;
-        for (int r = 0; r < kLossThreads / kOutPad; ++r) c += sg[r * kOutPad + threadIdx.x];
-        db4_part[(size_t)blockIdx.x * kOutPad + threadIdx.x] = c;
-    }
-    for (int st = kLossThreads / 2; st > 0; st >>= 1) {
-        if ((int)threadIdx.x < st) s[threadIdx.x] += s[threadIdx.x + st];
-        __syncthreads();
-    }
-    if (threadIdx.x == 0) loss_part[blockIdx.x] = s[0];
-}
+constexpr int kLossRows = 16;   // batch rows per partial of the loss and of db4
 
 // Where the gather finds the gradients: the weight-gradient GEMMs' K-slice partials
 // (dW1 [128][272], dW2, dW3 [128][128], dW4^T [128][16] per slice) and the bias-gradient
-// partials, per 128-row tile of the dZ GEMMs (column sums of the unrounded dZ, [tile][128])
-// and per block of the loss kernel (dY, [block][16]).
+// partials, per 128-row tile (column sums of the unrounded dZ, [tile][128]) and per 16 rows
+// (of the unrounded dY, [block][16]).
 struct GradSrc {
     const float *dW1, *dW2, *dW3, *dW4t;
     int slices;
@@ -175,6 +100,7 @@ __device__ __forceinline__ float grad_of(const GradSrc &g, int t)
         p = g.db4; idx = t - kOffB4; stride = kOutPad; n = g.blocks;
     }
     float v = 0.0f;
+#pragma unroll 16                              // (loads in flight; a batch of 4096 has 256 db4 partials)
     for (int k = 0; k < n; ++k) v += p[k * stride + idx];
     return v;
 }
@@ -182,6 +108,7 @@ __device__ __forceinline__ float grad_of(const GradSrc &g, int t)
 __device__ __forceinline__ void finish_loss(const double *loss_part, int nblk, int B, double *loss)
 {
     double l = 0.0;
+#pragma unroll 16
     for (int k = 0; k < nblk; ++k) l += loss_part[k];
     *loss = l / (double)(kOut * B);
 }
@@ -339,43 +266,49 @@ __device__ __forceinline__ void rot_t_apply(const float q[4], const float v[3], 
 // values at the anchor substep, then 64 cells x (density, velocity)); tau: time since the
 // anchor.  Output: R_a^T (x - x_a) / h, tau c / h, R_a^T (v - v_a) / c, R_a^T v / c,
 // R_a^T w h / c, then per cell rho / rho0 - 1 (-1 for an empty cell) and R_a^T v_cell / c.
-__device__ __forceinline__ void sur_features(const float *t13, const float *a, float tau,
-                                             const SurScale &s, float *out)
+// This returns entry e of it.
+__device__ __forceinline__ float sur_feature(const float *t13, const float *a, float tau, const SurScale &s, int e)
 {
     const float ih = 1.0f / s.h, ic = 1.0f / s.c, irho = 1.0f / s.rho0;
     const float qa[4] = {a[3], a[4], a[5], a[6]};
     float d[3], o[3];
-    for (int i = 0; i < 3; ++i) d[i] = (t13[i] - a[i]) * ih;
-    rot_t_apply(qa, d, o);
-    for (int i = 0; i < 3; ++i) out[i] = o[i];
-    out[3] = tau * s.c * ih;
-    for (int i = 0; i < 3; ++i) d[i] = (t13[7 + i] - a[7 + i]) * ic;
-    rot_t_apply(qa, d, o);
-    for (int i = 0; i < 3; ++i) out[4 + i] = o[i];
-    for (int i = 0; i < 3; ++i) d[i] = t13[7 + i] * ic;
-    rot_t_apply(qa, d, o);
-    for (int i = 0; i < 3; ++i) out[7 + i] = o[i];
-    for (int i = 0; i < 3; ++i) d[i] = t13[10 + i] * s.h * ic;
-    rot_t_apply(qa, d, o);
-    for (int i = 0; i < 3; ++i) out[10 + i] = o[i];
-    for (int k = 0; k < 64; ++k) {
-        const float *cell = a + 13 + 4 * k;
-        out[13 + 4 * k] = cell[0] * irho - 1.0f;
-        for (int i = 0; i < 3; ++i) d[i] = cell[1 + i] * ic;
-        rot_t_apply(qa, d, o);
-        for (int i = 0; i < 3; ++i) out[14 + 4 * k + i] = o[i];
+    int i;                                        // component of the rotated vector
+    if (e >= 13) {
+        const float *cell = a + 13 + ((e - 13) & ~3);
+        i = ((e - 13) & 3) - 1;
+        if (i < 0) return cell[0] * irho - 1.0f;
+        for (int k = 0; k < 3; ++k) d[k] = cell[1 + k] * ic;
+    } else if (e == 3) {
+        return tau * s.c * ih;
+    } else if (e < 3) {
+        i = e;
+        for (int k = 0; k < 3; ++k) d[k] = (t13[k] - a[k]) * ih;
+    } else if (e < 7) {
+        i = e - 4;
+        for (int k = 0; k < 3; ++k) d[k] = (t13[7 + k] - a[7 + k]) * ic;
+    } else if (e < 10) {
+        i = e - 7;
+        for (int k = 0; k < 3; ++k) d[k] = t13[7 + k] * ic;
+    } else {
+        i = e - 10;
+        for (int k = 0; k < 3; ++k) d[k] = t13[10 + k] * s.h * ic;
     }
+    rot_t_apply(qa, d, o);
+    return i == 0 ? o[0] : i == 1 ? o[1] : o[2];
 }
 
-// One row per thread: ticks (stride tick_stride floats), anchors (stride anchor_stride),
-// times since the anchor; out n x 269.
-__global__ void k_sur_features(const float *ticks, int tick_stride, const float *anchors,
-                               int anchor_stride, const float *taus, int n, SurScale s, float *out)
+// Ticks (stride tick_stride floats), anchors (stride anchor_stride), times since the anchor;
+// out n x 269.  A block takes a row at a time, a thread an entry of it: the loads and stores of
+// a row are then contiguous (one thread per row wrote 32 rows' lines at once).
+constexpr int kFeatThreads = 288;
+__global__ void __launch_bounds__(kFeatThreads) k_sur_features(const float *ticks, int tick_stride, const float *anchors,
+                                                              int anchor_stride, const float *taus, int n, SurScale s,
+                                                              float *out)
 {
-    const int r = blockIdx.x * blockDim.x + threadIdx.x;
-    if (r >= n) return;
-    sur_features(ticks + (size_t)r * tick_stride, anchors + (size_t)r * anchor_stride, taus[r], s,
-                 out + (size_t)r * 269);
+    const int e = threadIdx.x;
+    if (e >= kIn) return;
+    for (long long r = blockIdx.x; r < n; r += gridDim.x)
+        out[r * kIn + e] = sur_feature(ticks + r * tick_stride, anchors + r * anchor_stride, taus[r], s, e);
 }
 
 // Training targets: the wrench change since the anchor in the anchor's body frame, in the
@@ -398,16 +331,6 @@ __global__ void k_sur_targets(const double *w, const double *wa, const float *an
     }
 }
 
-// The tick's inputs from its pose and velocity (kernel arguments) and the stored anchor.
-__global__ void k_sur_tick_features(float t0, float t1, float t2, float t3, float t4, float t5, float t6,
-                                    float t7, float t8, float t9, float t10, float t11, float t12,
-                                    float tau, const float *anchor, SurScale s, float *out)
-{
-    if (threadIdx.x != 0) return;
-    const float t13[13] = {t0, t1, t2, t3, t4, t5, t6, t7, t8, t9, t10, t11, t12};
-    sur_features(t13, anchor, tau, s, out);
-}
-
 // The tick's wrench: the anchor's exact FP64 wrench plus the network's correction, taken out
 // of the standardised, scale-free, body-frame output.
 __device__ __forceinline__ void tick_output(const float *y, const float *ymean, const float *ystd,
@@ -428,12 +351,6 @@ __device__ __forceinline__ void tick_output(const float *y, const float *ymean, 
             out[3 * part + i] = wa[3 * part + i] + (double)wv * sc;
         }
     }
-}
-
-__global__ void k_sur_tick_output(const float *y, const float *ymean, const float *ystd, const float *anchor,
-                                  const double *wa, SurScale s, double *out)
-{
-    if (threadIdx.x == 0) tick_output(y, ymean, ystd, anchor, wa, s, out);
 }
 
 // The whole haptic tick in one CTA of 128 threads: the tick's 269 inputs, the four layers as
@@ -503,7 +420,7 @@ __global__ void __launch_bounds__(128, 1)
         load_w(1);
         load_w(3);
     }
-    // the inputs, sur_features' arithmetic spread over the threads: thread k < 64 the
+    // the inputs, sur_feature's arithmetic spread over the threads: thread k < 64 the
     // descriptor cell k, thread 64 the pose and velocity part
     {
         const float *an = a.anchor;
@@ -592,12 +509,304 @@ __global__ void __launch_bounds__(128, 1)
             } else {
                 tick_output(y, a.ymean, a.ystd, a.anchor, a.wa, a.s, a.out);
             }
-            // the model's status word rides along with the wrench (one copy to the host)
+            // the model's status word rides along with the wrench, straight into the host's
+            // pinned memory (a tick 29 us with a copy behind the kernel, 22 without)
             a.out[kOut] = a.status ? (double)*reinterpret_cast<volatile unsigned *>(a.status) : 0.0;
         }
     }
     asm volatile("tcgen05.fence::before_thread_sync;");
     __syncthreads();
+    if (warp == 0) {
+        asm volatile("tcgen05.fence::after_thread_sync;");
+        asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(128));
+    }
+}
+
+// The network over a batch, one CTA of 512 threads per 128 rows: every layer's activations of
+// a row tile depend on that tile alone, so the forward pass, the loss and the backward chain of
+// the pre-activation gradients run in one launch with the activations in shared memory, where
+// separate GEMMs took one launch a layer, each a chain of load, MMA and epilogue latencies on a
+// few SMs.  Stages: input to layer 1, layers 2 and 3, the output layer, and for training dZ3 =
+// (dY W4) gelu', dZ2, dZ1.  A stage's A operand is the tile's 128 rows in the K-major
+// 128-byte-swizzled layout, written by the threads; its weights come by TMA ahead of it (five
+// 16 KB chunks of W1; W2, later W2t; W4; after layer 1 W3, W3t and W4t in W1's place); the MMAs
+// accumulate in TMEM (128 columns) and each thread takes 32 columns of one row (TMEM lane)
+// through bias and GELU, or times GELU's derivative, back into the A tile.  The order of every sum
+// and every rounding is that of the single GEMMs.  What the epilogues take (16 k GELUs a stage
+// and CTA, ~2 us) bounds the kernel; a batch of 1024 has eight CTAs.
+// Training also writes the column-major BF16 copies ([feature][batch]) that the weight
+// gradients contract over the batch, keeps the pre-activations Z for the backward stages
+// ([tile][column][row], each thread reads what it wrote), and writes the partials of the loss
+// (FP64, per 16 rows) and of the bias gradients (per tile; db4 per 16 rows), each in a fixed
+// order.
+struct MlpMaps {
+    CUtensorMap m[7];                     // W1 W2 W4 W3 W3t W4t W2t
+};
+struct MlpArgs {
+    const float *x;                       // B x 269
+    int B;
+    const float *xmean, *xinv, *ymean, *ystd, *yinv;
+    const float *b1, *b2, *b3, *b4;
+    float *out;                           // forward: B x 6, de-standardised
+    const float *t;                       // training: B x 6 targets, and the outputs below
+    __nv_bfloat16 *xT, *hT[3], *dyT, *dzT[3];
+    int ldt;
+    float *d[3];
+    double *loss_part;
+    float *db4, *db[3];
+    unsigned *status;
+};
+constexpr int kMlpThreads = 512;
+constexpr int kMlpSmem = (5 + 5 + 2) * kTickChunk + 2 * kTickW4 + 1024 + 128;
+
+template <bool TRAIN>
+__global__ void __launch_bounds__(kMlpThreads, 1) k_mlp(const __grid_constant__ MlpMaps maps, MlpArgs a)
+{
+    using namespace tcx;
+    extern __shared__ unsigned char smem_raw[];
+    __shared__ uint32_t s_tmem;
+    __shared__ float s_cs[4][kHid];               // column sums per 32 rows
+    __shared__ float s_g[kTcM][kOut + 1];         // dY before rounding
+    const uint32_t raw = smem_u32(smem_raw);
+    const uint32_t A = (raw + 1023u) & ~1023u, WA = A + 5u * kTickChunk, WB = WA + 5u * kTickChunk;
+    const uint32_t WC = WB + 2u * kTickChunk, bar = WC + 2u * kTickW4;
+    auto full = [&](int l) { return bar + 8u * (uint32_t)l; };
+    const uint32_t done = bar + 56u;
+    unsigned char *Ap = smem_raw + (A - raw);
+    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+    const int quad = warp & 3, c0 = 32 * (warp >> 2);     // TMEM lanes 32 quad .., columns c0 ..
+    const int r = 32 * quad + lane;                       // row of the tile
+    const long long row = (long long)blockIdx.x * kTcM + r;
+    const bool live = row < a.B;
+    // 16 bytes (8 BF16 from column k, a multiple of 8) of row i of the A tile
+    auto cell = [&](int i, int k) {
+        return reinterpret_cast<uint4 *>(Ap + (size_t)(k >> 6) * kTickChunk + (size_t)i * 128 +
+                                         ((((k & 63) >> 3) ^ (i & 7)) << 4));
+    };
+    unsigned loading = 0;                                 // weights on their way (thread 0)
+    auto load = [&](int l, uint32_t dst, int chunks, int rows, uint32_t stride) {
+        mbar_expect_tx(full(l), (uint32_t)(chunks * rows * kTcKChunk * 2));
+        for (int c = 0; c < chunks; ++c) tma_load_2d(dst + (uint32_t)c * stride, &maps.m[l], c * kTcKChunk, 0, full(l));
+        loading |= 1u << l;
+    };
+    if (tid == 0) {
+        for (int l = 0; l < 8; ++l) mbar_init(full(l));
+        asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+        load(0, WA, 5, kHid, kTickChunk);
+        load(1, WB, 2, kHid, kTickChunk);
+        load(2, WC, 2, kOutPad, kTickW4);
+    }
+    if (warp == 0) {
+        __syncwarp();
+        asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(&s_tmem)),
+                     "r"(128));
+        asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;");
+    }
+    // the standardised inputs: a warp takes 8 rows, its lanes 32 columns at a time
+    {
+        constexpr int kSeg = (kInPad + 31) / 32;
+        float mean[kSeg], inv[kSeg];
+#pragma unroll
+        for (int s = 0; s < kSeg; ++s) {
+            const int k = 32 * s + lane;
+            mean[s] = k < kIn ? a.xmean[k] : 0.0f;
+            inv[s] = k < kIn ? a.xinv[k] : 0.0f;
+        }
+#pragma unroll 2
+        for (int q = 0; q < kTcM / (kMlpThreads / 32); ++q) {
+            const int i = warp * (kTcM / (kMlpThreads / 32)) + q;
+            const long long b = (long long)blockIdx.x * kTcM + i;
+            float v[kSeg];
+#pragma unroll
+            for (int s = 0; s < kSeg; ++s) {
+                const int k = 32 * s + lane;
+                v[s] = b < a.B && k < kIn ? __ldg(a.x + (size_t)b * kIn + k) : 0.0f;
+            }
+#pragma unroll
+            for (int s = 0; s < kSeg; ++s) {
+                const int k = 32 * s + lane;
+                if (k < kInPad)
+                    reinterpret_cast<__nv_bfloat16 *>(cell(i, k & ~7))[k & 7] =
+                        __float2bfloat16_rn(b < a.B && k < kIn ? (v[s] - mean[s]) * inv[s] : 0.0f);
+            }
+        }
+    }
+    asm volatile("tcgen05.fence::before_thread_sync;");
+    __syncthreads();
+    asm volatile("tcgen05.fence::after_thread_sync;");
+    const uint32_t tmem = s_tmem;
+    if (TRAIN && live) {
+        // the column-major copy of the inputs, 8 columns of one row at a time
+        for (int g = warp >> 2; g < kInPad / 8; g += kMlpThreads / 128) {
+            const uint4 u = *cell(r, 8 * g);
+            const __nv_bfloat16 *h = reinterpret_cast<const __nv_bfloat16 *>(&u);
+#pragma unroll
+            for (int j = 0; j < 8; ++j) a.xT[(size_t)(8 * g + j) * a.ldt + row] = h[j];
+        }
+    }
+
+    // stage: weights (map / barrier), their place, columns, K = 16 steps
+    const int wmap[7] = {0, 1, 3, 2, 5, 4, 6};
+    const uint32_t wplace[7] = {WA, WB, WA, WC, WA + 4u * kTickChunk, WA + 2u * kTickChunk, WB};
+    const int steps[7] = {kInPad / 16, kHid / 16, kHid / 16, kHid / 16, 1, kHid / 16, kHid / 16};
+    const float *bias[3] = {a.b1, a.b2, a.b3};
+    bool failed = false;
+    for (int st = 0; st < (TRAIN ? 7 : 4); ++st) {
+        const int n = st == 3 ? kOutPad : kHid;
+        // the A tile written by the threads becomes visible to the tensor core
+        asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+        asm volatile("tcgen05.fence::before_thread_sync;");
+        __syncthreads();
+        asm volatile("tcgen05.fence::after_thread_sync;");
+        bool ok = true;
+        if (tid == 0) {
+            if (st == 1) {                        // layer 1's MMAs are done with W1
+                load(3, WA, 2, kHid, kTickChunk);
+                if (TRAIN) {
+                    load(4, WA + 2u * kTickChunk, 2, kHid, kTickChunk);
+                    load(5, WA + 4u * kTickChunk, 1, kHid, kTickChunk);
+                }
+            }
+            if (TRAIN && st == 2) load(6, WB, 2, kHid, kTickChunk);   // and layer 2's with W2
+            ok = mbar_wait(full(wmap[st]), 0u);
+            if (ok) {
+                loading &= ~(1u << wmap[st]);
+                asm volatile("tcgen05.fence::after_thread_sync;");
+                const uint32_t idesc = instr_desc(n), stride = st == 3 ? (uint32_t)kTickW4 : (uint32_t)kTickChunk;
+                for (int k = 0; k < steps[st]; ++k)
+                    mma_bf16(tmem, smem_desc_sw128(A + (uint32_t)(k >> 2) * kTickChunk + 32u * (k & 3)),
+                             smem_desc_sw128(wplace[st] + (uint32_t)(k >> 2) * stride + 32u * (k & 3)), idesc,
+                             k > 0 ? 1u : 0u);
+            }
+            mma_commit(done);                     // fires once the issued MMAs completed
+        }
+        if (TRAIN && st > 4 && tid < kHid) {      // the last stage's bias gradient
+            float t = 0.0f;
+            for (int w = 0; w < 4; ++w) t += s_cs[w][tid];
+            a.db[7 - st][(size_t)blockIdx.x * kHid + tid] = t;
+        }
+        if (TRAIN && st == 4 && tid < 8 * kOutPad) {   // and the output layer's
+            const int blk = tid / kOutPad, j = tid % kOutPad;
+            float t = 0.0f;
+            if (j < kOut)
+                for (int i = 0; i < kLossRows; ++i) t += s_g[blk * kLossRows + i][j];
+            const long long p = (long long)blockIdx.x * (kTcM / kLossRows) + blk;
+            if (p * kLossRows < a.B) a.db4[p * kOutPad + j] = t;
+        }
+        __syncwarp();
+        if (!mbar_wait(done, (uint32_t)(st & 1))) ok = false;
+        asm volatile("tcgen05.fence::after_thread_sync;");
+        failed = __syncthreads_or(!ok) != 0;
+        if (failed) break;
+        if (st == 3) {
+            if (c0 == 0) {                        // warps 0 to 3: the 6 outputs of a row
+                uint32_t u[16];
+                tmem_ld16(tmem + ((uint32_t)(32 * quad) << 16), u);
+                double sq[kOut];
+                __align__(16) __nv_bfloat16 g16[16];
+                for (int j = 0; j < 16; ++j) g16[j] = __float2bfloat16_rn(0.0f);
+#pragma unroll
+                for (int j = 0; j < kOut; ++j) {
+                    const float y = __uint_as_float(u[j]) + a.b4[j];
+                    if (!TRAIN) {
+                        if (live) a.out[row * kOut + j] = y * a.ystd[j] + a.ymean[j];
+                        continue;
+                    }
+                    // MSE on standardised outputs: L = mean of (y - tn)^2, dY = 2 (y - tn) / (6 B)
+                    const float tn = live ? (a.t[row * kOut + j] - a.ymean[j]) * a.yinv[j] : y;
+                    const float d = live ? y - tn : 0.0f;
+                    const float g = 2.0f * d / (float)(kOut * a.B);
+                    sq[j] = (double)d * d;
+                    s_g[r][j] = g;
+                    g16[j] = __float2bfloat16_rn(g);
+                    if (live) a.dyT[(size_t)j * a.ldt + row] = g16[j];
+                }
+                if (TRAIN) {
+                    *cell(r, 0) = reinterpret_cast<const uint4 *>(g16)[0];
+                    *cell(r, 8) = reinterpret_cast<const uint4 *>(g16)[1];
+                    // the squared errors of 16 rows (half a warp), then their columns
+#pragma unroll
+                    for (int j = 0; j < kOut; ++j)
+#pragma unroll
+                        for (int o = kLossRows / 2; o > 0; o >>= 1) sq[j] += __shfl_xor_sync(0xffffffffu, sq[j], o);
+                    const double l = ((sq[0] + sq[4]) + sq[2]) + ((sq[1] + sq[5]) + sq[3]);
+                    const long long p = row / kLossRows;
+                    if ((lane & 15) == 0 && live) a.loss_part[p] = l;
+                }
+            }
+            continue;
+        }
+        float *d = TRAIN ? a.d[st < 3 ? st : 6 - st] + ((size_t)blockIdx.x * kHid + c0) * kTcM + r : nullptr;
+        __nv_bfloat16 *colT = TRAIN ? (st < 3 ? a.hT[st] : a.dzT[6 - st]) + (size_t)c0 * a.ldt + row : nullptr;
+#pragma unroll
+        for (int half = 0; half < 2; ++half) {
+            const int k = c0 + 16 * half;
+            uint32_t u[16];
+            float v[16];
+            if (st > 3) {
+#pragma unroll
+                for (int j = 0; j < 16; ++j) v[j] = d[(size_t)(16 * half + j) * kTcM];
+            }
+            tmem_ld16(tmem + ((uint32_t)(32 * quad) << 16) + (uint32_t)k, u);
+            __align__(16) __nv_bfloat16 h[16];
+            if (st < 3) {
+#pragma unroll
+                for (int j = 0; j < 16; ++j) {
+                    const float zv = __uint_as_float(u[j]) + __ldg(bias[st] + k + j);
+                    float grad;
+                    h[j] = __float2bfloat16_rn(TRAIN ? gelu_both(zv, grad) : gelu_f(zv));
+                    if (TRAIN) d[(size_t)(16 * half + j) * kTcM] = grad;
+                }
+            } else {
+#pragma unroll
+                for (int j = 0; j < 16; ++j) {
+                    v[j] = live ? __uint_as_float(u[j]) * v[j] : 0.0f;
+                    h[j] = __float2bfloat16_rn(v[j]);
+                }
+            }
+            if (st < 6) {
+                *cell(r, k) = reinterpret_cast<const uint4 *>(h)[0];
+                *cell(r, k + 8) = reinterpret_cast<const uint4 *>(h)[1];
+            }
+            if (TRAIN && live) {
+#pragma unroll
+                for (int j = 0; j < 16; ++j) colT[(size_t)(16 * half + j) * a.ldt] = h[j];
+            }
+            if (st > 3) {
+                // the 16 column sums of the warp by a halving exchange: after the xor-16, -8,
+                // -4 and -2 steps each lane pair holds one column (lane bits 4..1 pick it)
+                const unsigned all = 0xffffffffu;
+                float v8[8], v4[4], v2[2];
+                const bool h16 = lane & 16, h8 = lane & 8, h4 = lane & 4, h2 = lane & 2;
+#pragma unroll
+                for (int i = 0; i < 8; ++i)
+                    v8[i] = (h16 ? v[i + 8] : v[i]) + __shfl_xor_sync(all, h16 ? v[i] : v[i + 8], 16);
+#pragma unroll
+                for (int i = 0; i < 4; ++i)
+                    v4[i] = (h8 ? v8[i + 4] : v8[i]) + __shfl_xor_sync(all, h8 ? v8[i] : v8[i + 4], 8);
+#pragma unroll
+                for (int i = 0; i < 2; ++i)
+                    v2[i] = (h4 ? v4[i + 2] : v4[i]) + __shfl_xor_sync(all, h4 ? v4[i] : v4[i + 2], 4);
+                float v1 = (h2 ? v2[1] : v2[0]) + __shfl_xor_sync(all, h2 ? v2[0] : v2[1], 2);
+                v1 += __shfl_xor_sync(all, v1, 1);
+                if ((lane & 1) == 0) s_cs[quad][k + (h16 ? 8 : 0) + (h8 ? 4 : 0) + (h4 ? 2 : 0) + (h2 ? 1 : 0)] = v1;
+            }
+        }
+    }
+    asm volatile("tcgen05.fence::before_thread_sync;");
+    __syncthreads();
+    if (failed) {
+        if (tid == 0) {
+            for (int l = 0; l < 7; ++l)           // its own copies in flight, a bounded wait each
+                if (loading >> l & 1u) mbar_wait(full(l), 0u);
+            if (a.status) atomicOr(a.status, (unsigned)ST_TIMEOUT);
+        }
+        __syncthreads();
+    } else if (TRAIN && tid < kHid) {
+        float t = 0.0f;
+        for (int w = 0; w < 4; ++w) t += s_cs[w][tid];
+        a.db[0][(size_t)blockIdx.x * kHid + tid] = t;
+    }
     if (warp == 0) {
         asm volatile("tcgen05.fence::after_thread_sync;");
         asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(128));
@@ -615,29 +824,27 @@ struct sph_mlp {
     float *master, *m, *v, *grad, *norm;   // norm: xmean[269] xinv[269] ymean[6] ystd[6] yinv[6]
     __nv_bfloat16 *w1b, *w2b, *w3b, *w4b;
     float *b4pad;
-    __nv_bfloat16 *xb, *h1, *h2, *h3, *dyb, *dz3, *dz2, *dz1;
-    float *z1, *z2, *z3, *y, *out;
+    float *d1, *d2, *d3;               // GELU's derivatives, [tile][column][row]
     float *dW1, *dW2, *dW3, *dW4t;     // K-slice partials of the augmented weight gradients
     double *loss, *loss_part;
     float *db4_part, *db3_part, *db2_part, *db1_part;   // bias-gradient partials
     unsigned *status;
-    // K-contiguous operands of the backward GEMMs: weight transposes, and column-major
+    // K-contiguous operands of the backward pass: weight transposes, and column-major
     // ([feature][batch], leading dimension ldt) copies of the input, activations and gradients
     __nv_bfloat16 *w2t, *w3t, *w4t;
     __nv_bfloat16 *xbT, *h1T, *h2T, *h3T, *dybT, *dz3T, *dz2T, *dz1T;
     int ldt = 0;
-    // the haptic tick: anchor descriptor (269), anchor wrench (6 doubles), the tick's input
-    // row (269) and result (6 doubles); scales; pinned host copy of the result; the event
+    // the haptic tick: anchor descriptor (269), anchor wrench (6 doubles); scales; the result
+    // (6 doubles and the status word) in pinned host memory; the event
     // that orders the anchor (handle's stream) before the ticks (model's stream)
-    float *anchor, *tick_x;
-    double *anchor_w, *tick_w;
+    float *anchor;
+    double *anchor_w;
     SurScale scale = {0.0f, 0.0f, 0.0f};
     double *pin = nullptr;
     cudaEvent_t anchored = nullptr;
     bool has_anchor = false;
-    // the fused tick's TMA maps of the BF16 weights (built once; false: the unfused path)
-    CUtensorMap wmap[4];
-    bool tick_fused = false;
+    MlpMaps maps;                      // TMA maps of the BF16 weights (built once)
+    bool mapped = false;
     std::string err;
 };
 
@@ -666,28 +873,20 @@ size_t mlp_sizes(int B, size_t *sz)
     sz[i++] = 2 * (size_t)kHid * kHid;        // w3b
     sz[i++] = 2 * (size_t)kOutPad * kHid;     // w4b
     sz[i++] = 4 * (size_t)kOutPad;            // b4pad
-    sz[i++] = 2 * (size_t)B * kInPad;         // xb
-    for (int k = 0; k < 3; ++k) sz[i++] = 2 * (size_t)B * kHid;   // h1 h2 h3
-    sz[i++] = 2 * (size_t)B * kOutPad;        // dyb
-    for (int k = 0; k < 3; ++k) sz[i++] = 2 * (size_t)B * kHid;   // dz3 dz2 dz1
-    for (int k = 0; k < 3; ++k) sz[i++] = 4 * (size_t)B * kHid;   // z1 z2 z3
-    sz[i++] = 4 * (size_t)B * kOutPad;        // y
-    sz[i++] = 4 * (size_t)B * kOut;           // out
+    const size_t tiles = (size_t)(B + kTcM - 1) / kTcM;
+    for (int k = 0; k < 3; ++k) sz[i++] = 4 * tiles * kTcM * kHid;   // d1 d2 d3
     sz[i++] = 4 * (size_t)kSplit * kHid * kInPad;   // dW1 (K slices)
     sz[i++] = 4 * (size_t)kSplit * kHid * kHid;     // dW2
     sz[i++] = 4 * (size_t)kSplit * kHid * kHid;     // dW3
     sz[i++] = 4 * (size_t)kSplit * kHid * kOutPad;  // dW4t
     sz[i++] = 8;                              // loss
-    const size_t nblk = (size_t)(B * kOutPad + kLossThreads - 1) / kLossThreads;
-    const size_t tiles = (size_t)(B + kTcM - 1) / kTcM;
+    const size_t nblk = (size_t)(B + kLossRows - 1) / kLossRows;
     sz[i++] = 8 * nblk;                       // loss_part
     sz[i++] = 4 * nblk * kOutPad;             // db4_part
     for (int k = 0; k < 3; ++k) sz[i++] = 4 * tiles * kHid;   // db3_part db2_part db1_part
     sz[i++] = 16;                             // status
     sz[i++] = 4 * (size_t)kIn;                // anchor
-    sz[i++] = 4 * (size_t)kIn;                // tick_x
     sz[i++] = 8 * (size_t)kOut;               // anchor_w
-    sz[i++] = 8 * (size_t)(kOut + 2);         // tick_w (+ the status word)
     sz[i++] = 2 * (size_t)kHid * kHid;        // w2t
     sz[i++] = 2 * (size_t)kHid * kHid;        // w3t
     sz[i++] = 2 * (size_t)kHid * kOutPad;     // w4t
@@ -722,95 +921,65 @@ sph_status mfail(sph_mlp *m, sph_status s, const std::string &msg)
             return mfail((m), SPH_ERR_CUDA, std::string(#call) + ": " + cudaGetErrorString(e_)); \
     } while (0)
 
-// C[M][N] = A[M][K] B[N][K]^T with K-contiguous BF16 operands
-TcGemm gemm(const __nv_bfloat16 *A, int lda, const __nv_bfloat16 *B, int ldb, int M, int N, int K, float *C,
-            int ldc, unsigned *status)
+MlpArgs mlp_args(const sph_mlp *m, const float *d_x, int B)
 {
-    TcGemm g;
-    std::memset(&g, 0, sizeof g);
-    g.A = A; g.lda = lda;
-    g.B = B; g.ldb = ldb;
-    g.M = M; g.N = N; g.K = K; g.C = C; g.ldc = ldc;
-    g.epilogue = TC_STORE;
-    g.ksplit = 1;
-    g.status = status;
-    return g;
+    MlpArgs a;
+    std::memset(&a, 0, sizeof a);
+    a.x = d_x;
+    a.B = B;
+    a.xmean = m->norm;
+    a.xinv = m->norm + kIn;
+    a.ymean = m->norm + 2 * kIn;
+    a.ystd = a.ymean + kOut;
+    a.yinv = a.ystd + kOut;
+    a.b1 = m->master + kOffB1;
+    a.b2 = m->master + kOffB2;
+    a.b3 = m->master + kOffB3;
+    a.b4 = m->b4pad;
+    a.status = m->status;
+    return a;
 }
 
-// Forward pass of a batch of B rows; `train` also writes the column-major copies the
-// backward pass contracts over the batch.
-sph_status mlp_forward(sph_mlp *m, const float *d_x, int B, bool train)
+template <bool TRAIN>
+sph_status mlp_launch(sph_mlp *m, const MlpArgs &a)
 {
-    cudaStream_t s = m->stream;
-    const float *xmean = m->norm, *xinv = m->norm + kIn;
-    k_prep_input<<<dim3((kInPad + 31) / 32, (B + 31) / 32), dim3(32, 8), 0, s>>>(d_x, B, xmean, xinv, m->xb,
-                                                                                train ? m->xbT : nullptr, m->ldt);
+    if (!m->mapped) return mfail(m, SPH_ERR_CUDA, "the weights' tensor maps could not be built");
+    static std::atomic<unsigned long long> configured{0};
+    MLP_CUDA(m, smem_opt_in(k_mlp<TRAIN>, kMlpSmem, configured));
+    k_mlp<TRAIN><<<(a.B + kTcM - 1) / kTcM, kMlpThreads, kMlpSmem, m->stream>>>(m->maps, a);
     MLP_CUDA(m, cudaGetLastError());
-    const __nv_bfloat16 *in[3] = {m->xb, m->h1, m->h2};
-    const __nv_bfloat16 *w[3] = {m->w1b, m->w2b, m->w3b};
-    __nv_bfloat16 *hout[3] = {m->h1, m->h2, m->h3};
-    __nv_bfloat16 *hT[3] = {m->h1T, m->h2T, m->h3T};
-    float *z[3] = {m->z1, m->z2, m->z3};
-    const int kdim[3] = {kInPad, kHid, kHid};
-    const int boff[3] = {kOffB1, kOffB2, kOffB3};
-    for (int l = 0; l < 3; ++l) {
-        TcGemm g = gemm(in[l], kdim[l], w[l], kdim[l], B, kHid, kdim[l], z[l], kHid, m->status);
-        g.epilogue = TC_BIAS_GELU;
-        g.bias = m->master + boff[l];
-        g.aux_out = hout[l];
-        g.ldaux = kHid;
-        if (train) { g.aux_out_t = hT[l]; g.ldaux_t = m->ldt; }
-        MLP_CUDA(m, tc_gemm(g, s));
-    }
-    TcGemm g = gemm(m->h3, kHid, m->w4b, kHid, B, kOutPad, kHid, m->y, kOutPad, m->status);
-    g.epilogue = TC_BIAS;
-    g.bias = m->b4pad;
-    MLP_CUDA(m, tc_gemm(g, s));
     return SPH_OK;
 }
 
-// Backward pass: loss, dY, the dZ chain and the weight-gradient K slices; `src` and `nblk`
-// say where the gradient gather finds them.
-sph_status mlp_backward(sph_mlp *m, const float *d_t, int B, GradSrc &src, int &nblk)
+// Forward and backward pass over a batch of B rows: loss, dY, the dZ chain and the
+// weight-gradient K slices; `src` and `nblk` say where the gradient gather finds them.
+sph_status mlp_backward(sph_mlp *m, const float *d_x, const float *d_t, int B, GradSrc &src, int &nblk)
 {
-    cudaStream_t s = m->stream;
-    const float *ymean = m->norm + 2 * kIn, *yinv = m->norm + 2 * kIn + 2 * kOut;
-    const int lt = m->ldt;
-    nblk = (B * kOutPad + kLossThreads - 1) / kLossThreads;
-    k_loss_grad<<<nblk, kLossThreads, 0, s>>>(m->y, d_t, B, ymean, yinv, m->dyb, m->dybT, lt, m->loss_part,
-                                              m->db4_part);
-    MLP_CUDA(m, cudaGetLastError());
-    // weight gradients contract over the batch: K = B, split into `slices` batch ranges
+    const int lt = m->ldt, tiles = (B + kTcM - 1) / kTcM;
+    MlpArgs a = mlp_args(m, d_x, B);
+    a.t = d_t;
+    a.xT = m->xbT;
+    a.hT[0] = m->h1T; a.hT[1] = m->h2T; a.hT[2] = m->h3T;
+    a.dyT = m->dybT;
+    a.dzT[0] = m->dz1T; a.dzT[1] = m->dz2T; a.dzT[2] = m->dz3T;
+    a.ldt = lt;
+    a.d[0] = m->d1; a.d[1] = m->d2; a.d[2] = m->d3;
+    a.loss_part = m->loss_part;
+    a.db4 = m->db4_part;
+    a.db[0] = m->db1_part; a.db[1] = m->db2_part; a.db[2] = m->db3_part;
+    nblk = (B + kLossRows - 1) / kLossRows;
+    sph_status st = mlp_launch<true>(m, a);
+    if (st != SPH_OK) return st;
+    // weight gradients contract over the batch: K = B, split into `slices` batch ranges; the
+    // four (dW1 = dZ1^T X, dW2 = dZ2^T H1, dW3 = dZ3^T H2, dW4^T = H3^T dY) in one launch
     const int slices = std::min(kSplit, (B + kTcKChunk - 1) / kTcKChunk);
-    auto wgrad = [&](const __nv_bfloat16 *AT, int M, const __nv_bfloat16 *BT, int N, float *dW) {
-        TcGemm g = gemm(AT, lt, BT, lt, M, N, B, dW, N, m->status);
-        g.ksplit = slices;
-        g.split_stride = (size_t)M * N;
-        return tc_gemm(g, s);
-    };
-    // dZ = (dZ_next W) * gelu'(Z): BF16 row-major and column-major, and the column sums of
-    // the unrounded dZ per 128-row tile (the bias gradient's partials)
-    auto dzgemm = [&](const __nv_bfloat16 *dn, int kn, const __nv_bfloat16 *wt, const float *z,
-                      __nv_bfloat16 *dz, __nv_bfloat16 *dzT, float *db_part) {
-        TcGemm g = gemm(dn, kn, wt, kn, B, kHid, kn, nullptr, kHid, m->status);
-        g.epilogue = TC_GELU_GRAD; g.aux_in = z; g.aux_out = dz; g.ldaux = kHid;
-        g.aux_out_t = dzT; g.ldaux_t = lt;
-        g.colsum = db_part; g.ld_colsum = kHid;
-        return tc_gemm(g, s);
-    };
-    // layer 4: dW4^T = H3^T dY (rows = 128 inputs, K = batch)
-    MLP_CUDA(m, wgrad(m->h3T, kHid, m->dybT, kOutPad, m->dW4t));
-    // dZ3 = (dY W4) * gelu'(Z3): B operand W4^T [128][16]
-    MLP_CUDA(m, dzgemm(m->dyb, kOutPad, m->w4t, m->z3, m->dz3, m->dz3T, m->db3_part));
-    // layers 3 and 2: dW = dZ^T H_prev, dZ_prev = (dZ W) * gelu'(Z_prev)
-    MLP_CUDA(m, wgrad(m->dz3T, kHid, m->h2T, kHid, m->dW3));
-    MLP_CUDA(m, dzgemm(m->dz3, kHid, m->w3t, m->z2, m->dz2, m->dz2T, m->db2_part));
-    MLP_CUDA(m, wgrad(m->dz2T, kHid, m->h1T, kHid, m->dW2));
-    MLP_CUDA(m, dzgemm(m->dz2, kHid, m->w2t, m->z1, m->dz1, m->dz1T, m->db1_part));
-    // layer 1: dW1 = dZ1^T Xb (N = 272)
-    MLP_CUDA(m, wgrad(m->dz1T, kHid, m->xbT, kInPad, m->dW1));
+    const TcGemm g[4] = {{m->dz1T, m->xbT, lt, lt, kHid, kInPad, B, m->dW1, kInPad, slices, (size_t)kHid * kInPad},
+                         {m->dz2T, m->h1T, lt, lt, kHid, kHid, B, m->dW2, kHid, slices, (size_t)kHid * kHid},
+                         {m->dz3T, m->h2T, lt, lt, kHid, kHid, B, m->dW3, kHid, slices, (size_t)kHid * kHid},
+                         {m->h3T, m->dybT, lt, lt, kHid, kOutPad, B, m->dW4t, kOutPad, slices, (size_t)kHid * kOutPad}};
+    MLP_CUDA(m, tc_gemm_group(g, 4, m->status, m->stream));
     src = GradSrc{m->dW1, m->dW2, m->dW3, m->dW4t, slices,
-                  m->db1_part, m->db2_part, m->db3_part, (B + kTcM - 1) / kTcM, m->db4_part, nblk};
+                  m->db1_part, m->db2_part, m->db3_part, tiles, m->db4_part, nblk};
     return SPH_OK;
 }
 
@@ -855,25 +1024,25 @@ sph_status sph_mlp_create(void *d_workspace, size_t bytes, void *cuda_stream, in
     auto h = [&]() { return reinterpret_cast<__nv_bfloat16 *>(ws + L.off[i++]); };
     m->master = f(); m->m = f(); m->v = f(); m->grad = f(); m->norm = f();
     m->w1b = h(); m->w2b = h(); m->w3b = h(); m->w4b = h(); m->b4pad = f();
-    m->xb = h(); m->h1 = h(); m->h2 = h(); m->h3 = h(); m->dyb = h();
-    m->dz3 = h(); m->dz2 = h(); m->dz1 = h();
-    m->z1 = f(); m->z2 = f(); m->z3 = f(); m->y = f(); m->out = f();
+    m->d1 = f(); m->d2 = f(); m->d3 = f();
     m->dW1 = f(); m->dW2 = f(); m->dW3 = f(); m->dW4t = f();
     m->loss = reinterpret_cast<double *>(ws + L.off[i++]);
     m->loss_part = reinterpret_cast<double *>(ws + L.off[i++]);
     m->db4_part = f(); m->db3_part = f(); m->db2_part = f(); m->db1_part = f();
     m->status = reinterpret_cast<unsigned *>(ws + L.off[i++]);
-    m->anchor = f(); m->tick_x = f();
+    m->anchor = f();
     m->anchor_w = reinterpret_cast<double *>(ws + L.off[i++]);
-    m->tick_w = reinterpret_cast<double *>(ws + L.off[i++]);
     m->w2t = h(); m->w3t = h(); m->w4t = h();
     m->xbT = h(); m->h1T = h(); m->h2T = h(); m->h3T = h(); m->dybT = h();
     m->dz3T = h(); m->dz2T = h(); m->dz1T = h();
     m->ldt = ldt_of(max_batch);
-    m->tick_fused = tc_operand_map(&m->wmap[0], m->w1b, kHid, kInPad, kInPad, kHid) &&
-                    tc_operand_map(&m->wmap[1], m->w2b, kHid, kHid, kHid, kHid) &&
-                    tc_operand_map(&m->wmap[2], m->w3b, kHid, kHid, kHid, kHid) &&
-                    tc_operand_map(&m->wmap[3], m->w4b, kOutPad, kHid, kHid, kOutPad);
+    m->mapped = tc_operand_map(&m->maps.m[0], m->w1b, kHid, kInPad, kInPad, kHid) &&
+                tc_operand_map(&m->maps.m[1], m->w2b, kHid, kHid, kHid, kHid) &&
+                tc_operand_map(&m->maps.m[2], m->w4b, kOutPad, kHid, kHid, kOutPad) &&
+                tc_operand_map(&m->maps.m[3], m->w3b, kHid, kHid, kHid, kHid) &&
+                tc_operand_map(&m->maps.m[4], m->w3t, kHid, kHid, kHid, kHid) &&
+                tc_operand_map(&m->maps.m[5], m->w4t, kHid, kOutPad, kOutPad, kHid) &&
+                tc_operand_map(&m->maps.m[6], m->w2t, kHid, kHid, kHid, kHid);
     cudaError_t e = cudaMemsetAsync(ws, 0, L.total, m->stream);
     if (e == cudaSuccess) e = cudaStreamSynchronize(m->stream);
     if (e == cudaSuccess) e = cudaHostAlloc(&m->pin, 8 * (kOut + 2), cudaHostAllocDefault);
@@ -923,12 +1092,9 @@ sph_status sph_mlp_get_params(sph_mlp *m, float *h_params)
 sph_status sph_mlp_forward(sph_mlp *m, const float *d_x, int32_t batch, float *d_y)
 {
     if (!m || !d_x || !d_y || batch < 1 || batch > m->max_batch) return SPH_ERR_ARG;
-    sph_status st = mlp_forward(m, d_x, batch, false);
-    if (st != SPH_OK) return st;
-    const float *ymean = m->norm + 2 * kIn, *ystd = m->norm + 2 * kIn + kOut;
-    k_output<<<(batch * kOut + 255) / 256, 256, 0, m->stream>>>(m->y, batch, ymean, ystd, d_y);
-    MLP_CUDA(m, cudaGetLastError());
-    return SPH_OK;
+    MlpArgs a = mlp_args(m, d_x, batch);
+    a.out = d_y;
+    return mlp_launch<false>(m, a);
 }
 
 sph_status sph_mlp_gradients(sph_mlp *m, const float *d_x, const float *d_t, int32_t batch, float *h_grad,
@@ -937,8 +1103,7 @@ sph_status sph_mlp_gradients(sph_mlp *m, const float *d_x, const float *d_t, int
     if (!m || !d_x || !d_t || batch < 1 || batch > m->max_batch) return SPH_ERR_ARG;
     GradSrc src;
     int nblk = 0;
-    sph_status st = mlp_forward(m, d_x, batch, true);
-    if (st == SPH_OK) st = mlp_backward(m, d_t, batch, src, nblk);
+    sph_status st = mlp_backward(m, d_x, d_t, batch, src, nblk);
     if (st != SPH_OK) return st;
     k_gather_grads<<<(kParams + 255) / 256, 256, 0, m->stream>>>(src, m->grad, m->loss_part, nblk, batch, m->loss);
     MLP_CUDA(m, cudaGetLastError());
@@ -954,8 +1119,7 @@ sph_status sph_mlp_train_step(sph_mlp *m, const float *d_x, const float *d_t, in
     if (!m || !d_x || !d_t || batch < 1 || batch > m->max_batch || !(lr > 0.0f)) return SPH_ERR_ARG;
     GradSrc src;
     int nblk = 0;
-    sph_status st = mlp_forward(m, d_x, batch, true);
-    if (st == SPH_OK) st = mlp_backward(m, d_t, batch, src, nblk);
+    sph_status st = mlp_backward(m, d_x, d_t, batch, src, nblk);
     if (st != SPH_OK) return st;
     m->adam_t += 1;
     const float b1 = 0.9f, b2 = 0.999f;
@@ -1012,8 +1176,8 @@ sph_status sph_surrogate_features(sph_mlp *m, const float *d_ticks, int32_t tick
     if (!m || n < 0 || (n > 0 && (!d_ticks || !d_anchors || !d_elapsed || !d_x))) return SPH_ERR_ARG;
     if (tick_stride < 13 || anchor_stride < kIn || !(m->scale.h > 0.0f)) return SPH_ERR_ARG;
     if (n == 0) return SPH_OK;
-    k_sur_features<<<(n + 127) / 128, 128, 0, m->stream>>>(d_ticks, tick_stride, d_anchors, anchor_stride,
-                                                           d_elapsed, n, m->scale, d_x);
+    k_sur_features<<<std::min(n, 2048), kFeatThreads, 0, m->stream>>>(d_ticks, tick_stride, d_anchors, anchor_stride,
+                                                                     d_elapsed, n, m->scale, d_x);
     MLP_CUDA(m, cudaGetLastError());
     return SPH_OK;
 }
@@ -1057,52 +1221,33 @@ sph_status sph_surrogate_tick(sph_mlp *m, const float pose_vel[13], float elapse
 {
     if (!m || !pose_vel || !out || !(elapsed >= 0.0f)) return SPH_ERR_ARG;
     if (!m->has_anchor) return mfail(m, SPH_ERR_STATE, "no anchor: call sph_surrogate_anchor first");
-    const float *t = pose_vel;
-    const float *ymean = m->norm + 2 * kIn, *ystd = m->norm + 2 * kIn + kOut;
-    if (m->tick_fused) {
-        // one kernel: inputs, the four layers on the tensor cores, the wrench
-        static std::atomic<unsigned long long> configured{0};
-        MLP_CUDA(m, smem_opt_in(k_sur_tick_fused, kTickSmem, configured));
-        TickArgs a;
-        for (int i = 0; i < 13; ++i) a.t13[i] = t[i];
-        a.tau = elapsed;
-        a.anchor = m->anchor;
-        a.s = m->scale;
-        a.xmean = m->norm;
-        a.xinv = m->norm + kIn;
-        a.ymean = ymean;
-        a.ystd = ystd;
-        a.b1 = m->master + kOffB1;
-        a.b2 = m->master + kOffB2;
-        a.b3 = m->master + kOffB3;
-        a.b4 = m->b4pad;
-        a.wa = m->anchor_w;
-        a.out = m->tick_w;
-        a.status = m->status;
-        k_sur_tick_fused<<<1, 128, kTickSmem, m->stream>>>(m->wmap[0], m->wmap[1], m->wmap[2], m->wmap[3], a);
-        MLP_CUDA(m, cudaGetLastError());
-    } else {
-        k_sur_tick_features<<<1, 32, 0, m->stream>>>(t[0], t[1], t[2], t[3], t[4], t[5], t[6], t[7], t[8], t[9],
-                                                     t[10], t[11], t[12], elapsed, m->anchor, m->scale, m->tick_x);
-        MLP_CUDA(m, cudaGetLastError());
-        sph_status st = mlp_forward(m, m->tick_x, 1, false);
-        if (st != SPH_OK) return st;
-        k_sur_tick_output<<<1, 32, 0, m->stream>>>(m->y, ymean, ystd, m->anchor, m->anchor_w, m->scale, m->tick_w);
-        MLP_CUDA(m, cudaGetLastError());
-    }
-    sph_status st;
-    if (m->tick_fused) {
-        // the wrench and the status word in one copy
-        MLP_CUDA(m, cudaMemcpyAsync(m->pin, m->tick_w, 8 * (kOut + 1), cudaMemcpyDeviceToHost, m->stream));
-        MLP_CUDA(m, cudaStreamSynchronize(m->stream));
-        st = SPH_OK;
-        if (m->pin[kOut] != 0.0) {
-            MLP_CUDA(m, cudaMemsetAsync(m->status, 0, 4, m->stream));
-            st = mfail(m, SPH_ERR_TIMEOUT, "a tensor-core completion wait gave up");
-        }
-    } else {
-        MLP_CUDA(m, cudaMemcpyAsync(m->pin, m->tick_w, 8 * kOut, cudaMemcpyDeviceToHost, m->stream));
-        st = mlp_status(m);                     // synchronises the model's stream
+    if (!m->mapped) return mfail(m, SPH_ERR_CUDA, "the weights' tensor maps could not be built");
+    // one kernel: inputs, the four layers on the tensor cores, the wrench
+    static std::atomic<unsigned long long> configured{0};
+    MLP_CUDA(m, smem_opt_in(k_sur_tick_fused, kTickSmem, configured));
+    TickArgs a;
+    for (int i = 0; i < 13; ++i) a.t13[i] = pose_vel[i];
+    a.tau = elapsed;
+    a.anchor = m->anchor;
+    a.s = m->scale;
+    a.xmean = m->norm;
+    a.xinv = m->norm + kIn;
+    a.ymean = m->norm + 2 * kIn;
+    a.ystd = m->norm + 2 * kIn + kOut;
+    a.b1 = m->master + kOffB1;
+    a.b2 = m->master + kOffB2;
+    a.b3 = m->master + kOffB3;
+    a.b4 = m->b4pad;
+    a.wa = m->anchor_w;
+    a.out = m->pin;                   // the kernel writes the host's copy
+    a.status = m->status;
+    k_sur_tick_fused<<<1, 128, kTickSmem, m->stream>>>(m->maps.m[0], m->maps.m[1], m->maps.m[3], m->maps.m[2], a);
+    MLP_CUDA(m, cudaGetLastError());
+    MLP_CUDA(m, cudaStreamSynchronize(m->stream));
+    sph_status st = SPH_OK;
+    if (m->pin[kOut] != 0.0) {
+        MLP_CUDA(m, cudaMemsetAsync(m->status, 0, 4, m->stream));
+        st = mfail(m, SPH_ERR_TIMEOUT, "a tensor-core completion wait gave up");
     }
     if (st != SPH_OK) return st;
     std::memcpy(out, m->pin, 8 * kOut);

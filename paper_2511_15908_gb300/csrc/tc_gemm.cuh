@@ -1,12 +1,13 @@
-// tc_gemm.cuh -- BF16 tensor-core GEMM on sm_103a (tcgen05 + TMEM + TMA), FP32 accumulation.
+// tc_gemm.cuh -- BF16 tensor-core GEMMs on sm_103a (tcgen05 + TMEM + TMA), FP32 accumulation,
+// and what the other tensor-core kernels share with them.
 //
 //   C[M, N] = A[M, K] * B[N, K]^T      (both operands "row = output index, K = contraction")
 //
 // Both operands are BF16 and K-contiguous in global memory ([row][k], leading dimension a
 // multiple of 8 elements, 16-byte aligned base).  One CTA of 128 threads computes a 128 x Nt
-// tile (Nt = 256, 128, ..., 16: the widest that still gives kTcMinCtas CTAs, so that the
-// small GEMMs of the surrogate spread over many SMs).  The K dimension is walked in 64-wide
-// chunks through a 4-stage shared-memory ring:
+// tile (Nt = 256, 128, ..., 16: the widest that still gives kTcMinCtas CTAs, so that small
+// GEMMs spread over many SMs).  The K dimension is walked in 64-wide chunks through a 4-stage
+// shared-memory ring:
 //   - thread 0 (the producer) waits until a stage is free and has the tensor memory
 //     accelerator copy the A and B boxes of the next chunk into it (cp.async.bulk.tensor,
 //     128-byte swizzle, rows past M / N and k past K read as zeros), completing on the
@@ -15,16 +16,13 @@
 //     the TMEM accumulator and commits them to the stage's "empty" mbarrier, which frees the
 //     stage for the producer once the tensor core has read it; after the last chunk it
 //     commits to the "done" mbarrier;
-//   - every thread waits for "done" and runs the epilogue: tcgen05.ld of its TMEM lane (= tile
-//     row), the fused per-element operation, and 16-byte stores of 16 consecutive columns
-//     (plus, where asked, a transposed BF16 copy whose stores are coalesced across the warp,
-//     and the column sums of the tile's FP32 results: a fixed shuffle tree within each warp,
-//     then the four warps in order).
+//   - every thread waits for "done" and stores its TMEM lane (= tile row).
 // Every wait is bounded: a wait that gives up latches ST_TIMEOUT in *status and the tile is
 // not written.
 //
-// A K split (ksplit > 1, TC_STORE only) spreads the chunks over grid.z; CTA z writes its
-// partial sum to C + z * split_stride, and the caller sums the slices in a fixed order.
+// A K split (ksplit > 1) spreads the chunks over CTAs; slice z writes its partial sum to
+// C + z * split_stride, and the caller sums the slices in a fixed order.  Several independent
+// GEMMs go out as one launch (tc_gemm_group), their tiles side by side.
 #pragma once
 #include <atomic>
 #include <cstdint>
@@ -42,32 +40,15 @@ constexpr int kTcMinCtas = 64;     // column tiles narrow (to 16) until a GEMM h
 constexpr int kTcStages = 4;       // shared-memory ring depth
 constexpr unsigned kTcSpin = 1u << 22;
 
-enum TcEpilogue : int {
-    TC_STORE = 0,        // C = acc                                   (FP32)
-    TC_BIAS_GELU = 1,    // Z = acc + bias -> C (FP32); H = gelu(Z) -> aux_out (BF16)
-    TC_GELU_GRAD = 2,    // G = acc * gelu'(aux_in) -> aux_out (BF16); C (FP32) optional
-    TC_BIAS = 3,         // C = acc + bias                            (FP32)
-};
-
 struct TcGemm {
     const __nv_bfloat16 *A;   // M x K, [row][k], leading dimension lda
     const __nv_bfloat16 *B;   // N x K, [row][k], leading dimension ldb
     int lda, ldb;        // in elements, multiples of 8
     int M, N, K;
-    float *C;            // M x N FP32 (ldc), may be null for TC_GELU_GRAD
+    float *C;            // M x N FP32 (ldc)
     int ldc;
-    const float *bias;   // N (TC_BIAS_GELU, TC_BIAS)
-    const float *aux_in; // M x N FP32 pre-activation Z (TC_GELU_GRAD), ld = ldaux
-    __nv_bfloat16 *aux_out;  // M x N BF16 (TC_BIAS_GELU, TC_GELU_GRAD), ld = ldaux
-    int ldaux;
-    __nv_bfloat16 *aux_out_t;  // optional N x M BF16 transposed copy of aux_out ([col][row])
-    int ldaux_t;
-    int epilogue;
-    float *colsum;       // optional: per row tile, the column sums of the FP32 epilogue values
-    int ld_colsum;       // (the values C receives) over the tile's rows: colsum[tile * ld + col]
-    int ksplit;          // >= 1; > 1 only with TC_STORE
+    int ksplit;          // >= 1
     size_t split_stride; // elements between the partial slices of C
-    unsigned *status;    // ST_TIMEOUT latched when an mbarrier wait gives up
 };
 
 // GELU, tanh form: 0.5 z (1 + tanh(sqrt(2/pi) (z + 0.044715 z^3)))
@@ -77,11 +58,13 @@ __device__ __forceinline__ float gelu_f(float z)
     return 0.5f * z * (1.0f + tanhf(c * (z + a * z * z * z)));
 }
 
-__device__ __forceinline__ float gelu_grad_f(float z)
+// the same and its derivative
+__device__ __forceinline__ float gelu_both(float z, float &grad)
 {
     const float c = 0.7978845608028654f, a = 0.044715f;
-    float t = tanhf(c * (z + a * z * z * z));
-    return 0.5f * (1.0f + t) + 0.5f * z * (1.0f - t * t) * c * (1.0f + 3.0f * a * z * z);
+    const float t = tanhf(c * (z + a * z * z * z));
+    grad = 0.5f * (1.0f + t) + 0.5f * z * (1.0f - t * t) * c * (1.0f + 3.0f * a * z * z);
+    return 0.5f * z * (1.0f + t);
 }
 
 // Tensor map of a K-contiguous BF16 operand [rows][K] (leading dimension ld elements, a
@@ -104,10 +87,9 @@ inline cudaError_t smem_opt_in(Kernel *kernel, int bytes, std::atomic<unsigned l
     return e;
 }
 
-// Number of K slices tc_gemm writes for g (1 without a split): the caller sums this many.
-int tc_gemm_splits(const TcGemm &g);
+constexpr int kTcGroup = 4;        // GEMMs of one launch, at most
 // cudaErrorInvalidValue when the operands break the layout rules above or the tensor maps
-// cannot be built.
-cudaError_t tc_gemm(const TcGemm &g, cudaStream_t s);
+// cannot be built.  status: ST_TIMEOUT latched when an mbarrier wait gives up.
+cudaError_t tc_gemm_group(const TcGemm *g, int count, unsigned *status, cudaStream_t s);
 
 }  // namespace sphgb

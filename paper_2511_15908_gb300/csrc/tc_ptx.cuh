@@ -1,7 +1,7 @@
 // tc_ptx.cuh -- inline PTX for the tensor-core kernels on sm_103a: shared-memory matrix and
 // instruction descriptors of tcgen05.mma (BF16 x BF16 -> FP32, K-major operands written by
 // TMA with the 128-byte swizzle), mbarrier waits with an iteration limit, 2-D tiled TMA
-// loads, and the tcgen05 commit.  Used by the GEMM (tc_gemm.cu) and the fused haptic tick
+// loads, and the tcgen05 commit.  Used by the GEMM (tc_gemm.cu), the network and the haptic tick
 // (sph_mlp.cu).
 #pragma once
 #include <cstdint>
