@@ -204,7 +204,11 @@ bool iso_grid(const float lo[3], const float hi[3], float a, IsoGrid &g)
     return (double)g.n[0] * g.n[1] * g.n[2] < 2.0e9;
 }
 
-// Field of the fluid particles at every corner: sum over fluid j within 2h of m_j W.
+// Field of the fluid particles at every corner: sum over fluid j within 2h of m_j W, one thread
+// per corner.  Four candidates at a time overlap their loads where few warps have any (sort and
+// field, us: 156,816 corners 166 -> 144, 650,475 165 -> 150), but cost more past the rows' ends
+// than they hide on the largest grids (1,994,652: 274 -> 294).
+template <int U>
 __global__ void __launch_bounds__(kTile) k_iso_field(SimConst c, IsoGrid g, float *field)
 {
     const long long v = (long long)blockIdx.x * blockDim.x + threadIdx.x;
@@ -219,17 +223,113 @@ __global__ void __launch_bounds__(kTile) k_iso_field(SimConst c, IsoGrid g, floa
     DensitySum acc;
     uint32_t bad = 0;
     for_each_row(c, p, bad, [&](int s0, int e0) {
-        for (int q = s0; q < e0; ++q) {
-            const float4 xj = __ldg(c.xA + q);
-            if (!(xj.w > 0.0f)) continue;                   // boundary particle
-            float dx, dy, dz;
-            const float r2 = dist2(p, xj, dx, dy, dz);
-            if (!(r2 < c.R2)) continue;
-            if (__float_as_int(__ldg(vw + 4 * (size_t)q)) >= c.nf) continue;   // soft body
-            acc.add(c, xj, r2);
+        // U candidates' loads at a time, past the range's end too (xA is followed by vA in the
+        // workspace)
+        for (int q0 = s0; q0 < e0; q0 += U) {
+            float4 xs[U];
+            float r2[U];
+            bool in[U];
+#pragma unroll
+            for (int u = 0; u < U; ++u) xs[u] = __ldg(c.xA + q0 + u);
+#pragma unroll
+            for (int u = 0; u < U; ++u) {
+                float dx, dy, dz;
+                r2[u] = dist2(p, xs[u], dx, dy, dz);
+                in[u] = q0 + u < e0 && xs[u].w > 0.0f && r2[u] < c.R2;    // (a boundary particle's w < 0)
+            }
+#pragma unroll
+            for (int u = 0; u < U; ++u)                                   // not of a soft body
+                in[u] = in[u] && __float_as_int(__ldg(vw + 4 * (size_t)(q0 + u))) < c.nf;
+#pragma unroll
+            for (int u = 0; u < U; ++u)
+                if (in[u]) acc.add(c, xs[u], r2[u]);
         }
     });
     field[v] = __fmaf_rn(c.alpha6_hi, acc.S, c.alpha6_lo * acc.S - c.alpha6_hi * acc.C);
+}
+
+// The same sum, bit for bit, with G lanes per corner: the lanes set up the corner's rows
+// together, test G candidates at a time and compute their terms, which every lane then takes
+// into the compensated sum in the order of the walk (a ballot gives each its place in a queue in
+// shared memory).  A corner inside the fluid has some 270 neighbours and twice as many
+// candidates, for a single thread one chain of loads.  The whole warp calls this.
+template <int G>
+struct CornerWork {
+    CoopRows rows;
+    float terms[2 * G];
+};
+template <int G>
+__device__ __forceinline__ float iso_corner(const SimConst &c, float4 p, bool live, CornerWork<G> &s)
+{
+    constexpr unsigned kAll = 0xffffffffu;
+    const int l = threadIdx.x & (G - 1), gbase = threadIdx.x & 31 & ~(G - 1);
+    const float *vw = reinterpret_cast<const float *>(c.vA) + 3;   // id bits, stride 4
+    const unsigned lt = (1u << l) - 1u;
+    int longest, queued = 0;
+    const int nrows = coop_rows<G>(c, p, live, s.rows, longest);
+    DensitySum acc;
+    const int nr = __reduce_max_sync(kAll, nrows);
+    for (int r = 0; r < nr; ++r) {
+        const int2 e = r < nrows ? s.rows.row[r] : make_int2(0, 0);
+        for (int t = l; __any_sync(kAll, t - l < e.y); t += G) {
+            const int q = e.x + t;
+            bool in = t < e.y;
+            float m = 0.0f, r2 = 0.0f;
+            if (in) {
+                const float4 xj = __ldg(c.xA + q);
+                float dx, dy, dz;
+                r2 = dist2(p, xj, dx, dy, dz);
+                m = xj.w;                                   // (a boundary particle's is negative)
+                in = m > 0.0f && r2 < c.R2 && __float_as_int(__ldg(vw + 4 * (size_t)q)) < c.nf;
+            }
+            const unsigned found = __ballot_sync(kAll, in) >> gbase & group_mask<G>();
+            if (in) s.terms[queued + __popc(found & lt)] = DensitySum::term(c, m, r2);
+            queued += __popc(found);
+            __syncwarp();
+            if (__any_sync(kAll, queued >= G)) {
+                const bool take = queued >= G;
+                if (take) {
+#pragma unroll
+                    for (int u = 0; u < G; ++u) acc.add_term(s.terms[u]);
+                }
+                __syncwarp();
+                const float rest = s.terms[G + l];
+                __syncwarp();
+                if (take) {
+                    s.terms[l] = rest;
+                    queued -= G;
+                }
+                __syncwarp();
+            }
+        }
+    }
+    for (int u = 0; u < queued; ++u) acc.add_term(s.terms[u]);
+    __syncwarp();
+    return __fmaf_rn(c.alpha6_hi, acc.S, c.alpha6_lo * acc.S - c.alpha6_hi * acc.C);
+}
+
+__device__ __forceinline__ float4 corner_at(const IsoGrid &g, long long v)
+{
+    const int i = (int)(v % g.n[0]);
+    const int j = (int)((v / g.n[0]) % g.n[1]);
+    const int k = (int)(v / ((long long)g.n[0] * g.n[1]));
+    return make_float4(__fmaf_rn((float)i, g.a, g.o[0]), __fmaf_rn((float)j, g.a, g.o[1]),
+                       __fmaf_rn((float)k, g.a, g.o[2]), 0.0f);
+}
+
+// Small grids only.  The field with the sort before it, us, one thread / 8 lanes a corner: 18,009
+// corners 154 / 102, 78,416 153 / 109, 130,500 151 / 126, 156,816 166 / 142, 650,475 165 / 328: a
+// large grid is mostly air, where the lanes find nothing to share (4 lanes 230 there and 114 at
+// 18,009; 16 lanes 532 and 88; lanes for the corners with candidates only, found first by one
+// thread each, 291).
+template <int G>
+__global__ void __launch_bounds__(kTile) k_iso_field_lanes(SimConst c, IsoGrid g, float *field)
+{
+    __shared__ CornerWork<G> s[kTile / G];
+    const long long v = (long long)blockIdx.x * (kTile / G) + threadIdx.x / G;
+    const bool live = v < (long long)g.n[0] * g.n[1] * g.n[2];
+    const float f = iso_corner<G>(c, corner_at(g, live ? v : 0), live, s[threadIdx.x / G]);
+    if (live && (threadIdx.x & (G - 1)) == 0) field[v] = f;
 }
 
 struct IsoCubes {
@@ -364,6 +464,9 @@ bool iso_layout(const int32_t dims[3], IsoLayout &L)
     return true;
 }
 
+constexpr int kIsoLanes = 8;                       // (figures at k_iso_field_lanes)
+constexpr long long kIsoLanesMax = 160000, kIsoFourMax = 800000;
+
 unsigned blocks(long long n) { return (unsigned)((n + kTile - 1) / kTile); }
 
 }  // namespace
@@ -404,7 +507,10 @@ sph_status sph_iso_field(sph_handle *h, float cube, float *d_field)
         if (cudaMemsetAsync(d_field, 0, 4 * (size_t)nv, s) != cudaSuccess) return SPH_ERR_CUDA;
         return SPH_OK;
     }
-    k_iso_field<<<blocks(nv), kTile, 0, s>>>(c, g, d_field);
+    if (nv <= kIsoLanesMax && c.Rc < 2.5f)         // (the cooperative walk's row table)
+        k_iso_field_lanes<kIsoLanes><<<blocks(nv * kIsoLanes), kTile, 0, s>>>(c, g, d_field);
+    else
+        (nv <= kIsoFourMax ? k_iso_field<4> : k_iso_field<1>)<<<blocks(nv), kTile, 0, s>>>(c, g, d_field);
     return cudaGetLastError() == cudaSuccess ? SPH_OK : SPH_ERR_CUDA;
 }
 
