@@ -15,11 +15,11 @@
 #define SPH_DENSITY_MINB 4
 #define SPH_FORCE_MINB 6
 #define SPH_FORCE_COOP_MINB 3
-// Low-latency density pass (SPH_FLAG_LOW_LATENCY): G lanes per particle, 32 up to
-// kLowLatency32Max particles, else 16.  Measured (density pass, us) on the dam break (12k
-// particles) / a compact stirring tank (4.8k) / the coupled scene with 60k fluid (83k):
-// one thread 129 / 94 / 154; G = 4: 148 / 81 / 205; G = 8: 67 / 37 / 109; G = 16: 34 / 22
-// / 94; G = 32: 25 / 16 / 111 (4 resident blocks; 3 and 2 the same).
+// Low-latency density pass (SPH_FLAG_LOW_LATENCY): up to kLowLatency32Max particles 32 lanes each
+// that walk over the candidates, above 16 lanes that sum over the search's list.  Walking (us)
+// on the dam break (12k particles) / a compact stirring tank (4.8k) / the coupled scene with 60k
+// fluid (83k): G = 8: 67 / 37 / 109; G = 16: 34 / 22 / 94; G = 32: 25 / 16 / 111 (4 resident
+// blocks; 3 and 2 the same).  Search and list sums: dam break 28 (32 lanes), coupled 75 (16).
 #ifndef SPH_LOW_LATENCY_MINB
 #define SPH_LOW_LATENCY_MINB 4
 #endif
@@ -51,9 +51,14 @@ __global__ void __launch_bounds__(SPH_SEARCH_THREADS, SPH_SEARCH_MINB) k_search(
     search_item<SPH_SEARCH_THREADS, COOP>(c, blockIdx.x);
 }
 template <int G>
-__global__ void __launch_bounds__(kTile, SPH_LOW_LATENCY_MINB) k_density_coop(SimConst c)
+__global__ void __launch_bounds__(kTile, SPH_LOW_LATENCY_MINB) k_density_walk(SimConst c)
 {
-    density_coop_item<G>(c, blockIdx.x);
+    density_walk_item<G>(c, blockIdx.x);
+}
+template <int G>
+__global__ void __launch_bounds__(kTile, SPH_LOW_LATENCY_MINB) k_density_lanes(SimConst c)
+{
+    density_lanes_item<G>(c, blockIdx.x);
 }
 __global__ void __launch_bounds__(kTile) k_boundary_volume(SimConst c) { boundary_volume_item(c, blockIdx.x); }
 template <bool VOL>
@@ -186,16 +191,16 @@ cudaError_t launch_substep(const SimConst &c, cudaStream_t s, cudaEvent_t *ev, b
     k_rank_gather<<<nb, kTile, 0, s>>>(c);
     mark();
     // the neighbour search and the sums over its lists (timed together); the volume variant's
-    // boundary weights between them.  The low-latency pass searches for itself; its group's
-    // rows fit its 6 x 6 table while Rc < 2.5 (cells >= h give Rc ~ 2)
-    if ((c.flags & FLAG_LOW_LATENCY) && !(c.flags & FLAG_VOLUME) && c.Rc < 2.5f) {
-        if (c.n <= kLowLatency32Max)
-            k_density_coop<32><<<(unsigned)(((long long)c.n * 32 + kTile - 1) / kTile), kTile, 0, s>>>(c);
-        else
-            k_density_coop<16><<<(unsigned)(((long long)c.n * 16 + kTile - 1) / kTile), kTile, 0, s>>>(c);
+    // boundary weights between them.  The low-latency pass's walk has rows for Rc < 2.5 (cells >= h
+    // give Rc ~ 2)
+    const bool lanes = (c.flags & FLAG_LOW_LATENCY) && !(c.flags & FLAG_VOLUME) && c.Rc < 2.5f, walk = lanes && c.n <= kLowLatency32Max;
+    const auto search = c.coop == 0 ? k_search<0> : c.coop == 1 ? k_search<1> : k_search<2>;
+    if (!walk) search<<<search_tiles(c, SPH_SEARCH_THREADS), SPH_SEARCH_THREADS, 0, s>>>(c);
+    if (walk) {
+        k_density_walk<32><<<(unsigned)tiles_of<32>(c.n, kTile), kTile, 0, s>>>(c);
+    } else if (lanes) {
+        k_density_lanes<16><<<(unsigned)tiles_of<16>(c.n, kTile), kTile, 0, s>>>(c);
     } else {
-        const auto search = c.coop == 0 ? k_search<0> : c.coop == 1 ? k_search<1> : k_search<2>;
-        search<<<search_tiles(c, SPH_SEARCH_THREADS), SPH_SEARCH_THREADS, 0, s>>>(c);
         const bool vol = (c.flags & FLAG_VOLUME) != 0;
         if (vol && c.n > c.nf) k_boundary_volume<<<blocks_for(c.n - c.nf, kTile), kTile, 0, s>>>(c);
         const auto density = vol ? (c.coop == 0 ? k_density<0, DENSITY_VOLUME> : c.coop == 1 ? k_density<1, DENSITY_VOLUME> : k_density<2, DENSITY_VOLUME>)
