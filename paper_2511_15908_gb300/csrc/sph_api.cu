@@ -72,7 +72,8 @@ Layout make_layout(const sph_params &p, const sph_capacity &cap)
     L.n_scan_tiles = (L.ncell + kScanTile - 1) / kScanTile;
     const size_t N = (size_t)std::max(cap.max_particles, 1);
     L.max_wblocks = (int)((N + kReduceChunk - 1) / kReduceChunk) + kMaxBodies;
-    L.max_force_blocks = (int)((N + kForceThreads - 1) / kForceThreads);
+    L.max_force_blocks = (int)std::max((N + kForceThreads - 1) / kForceThreads,
+                                       (std::min<size_t>(N, kForceOrderedMax) * kForceOrderedG + 255) / 256);
     // the low-latency force pass writes a diagnostic row per block of 256 / G particles
     if ((p.flags & SPH_FLAG_LOW_LATENCY) && !(p.flags & SPH_FLAG_VOLUME_BOUNDARY))
         L.max_force_blocks = (int)((N * kLowLatencyForceG + 255) / 256);
@@ -244,9 +245,7 @@ sph_status finalize(sph_handle *h)
     for (const DevBody &B : h->bodies)
         if (B.kind == SPH_BODY_RIGID) c.n_rigid += B.n;
     c.coop = walk_coop(c);
-    c.n_force_blocks = (n + kForceThreads - 1) / kForceThreads;
-    if ((h->p.flags & SPH_FLAG_LOW_LATENCY) && !(h->p.flags & SPH_FLAG_VOLUME_BOUNDARY))
-        c.n_force_blocks = (int)(((long long)n * kLowLatencyForceG + 255) / 256);
+    c.n_force_blocks = force_blocks(c);
     for (int b = 0; b < kMaxBodies; ++b) {
         c.body_end[b] = b < c.nb ? h->bodies[b].first + h->bodies[b].n : n;
         c.body_kind[b] = b < c.nb ? h->bodies[b].kind : 0;

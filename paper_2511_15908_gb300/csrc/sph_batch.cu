@@ -317,7 +317,7 @@ cudaError_t launch_branches(sph_batch *b, int n_substeps, int cycle_end)
             e = cudaStreamWaitEvent(b->branch[k], b->fork, 0);
         for (int sc = 0; e == cudaSuccess && sc < b->n; ++sc) {
             SimConst c = b->table[sc];
-            c.n_force_blocks = (c.n + kForceThreads - 1) / kForceThreads;   // launched alone
+            c.n_force_blocks = force_blocks(c);             // launched alone
             for (int i = 0; e == cudaSuccess && i < n_substeps; ++i)
                 e = launch_substep(c, b->branch[b->branch_of[sc]]);
         }

@@ -22,6 +22,10 @@ constexpr int kMaxCell = 512;       // particles per cell for the deterministic 
 #endif
 constexpr int kLowLatencyForceG = SPH_LOW_LATENCY_FORCE_G;
 constexpr int kForceThreads = 128;  // particles per block (and diagnostic row) of the force pass
+// Scenes of at most kForceOrderedMax particles whose walk cooperates throughout (SimConst::coop
+// 2): the force pass takes kForceOrderedG lanes per particle (dam break, 12k particles: 20.5 us
+// with one thread each, 12.3 with the lanes; from 29k on they gain nothing: 20.5 / 22.5).
+constexpr int kForceOrderedG = 8, kForceOrderedMax = 20000;
 constexpr int kScanTile = 2048;     // cells per scan block (256 threads x 8)
 constexpr int kReduceChunk = 256;   // body particles per wrench-reduction block
 constexpr int kWrenchMinBlocks = 128; // the FP64 reduction is spread over at least this many
@@ -121,6 +125,8 @@ cudaError_t launch_substep(const SimConst &c, cudaStream_t s, cudaEvent_t *ev = 
                            unsigned ev_mask = ~0u);
 // who walks with cooperating lanes in a scene stepped alone
 int walk_coop(const SimConst &c);
+// blocks (and diagnostic rows) of the force pass of a scene stepped alone
+int force_blocks(const SimConst &c);
 // the events around the density pass alone (events 5 and 6)
 constexpr unsigned kDensityEvents = (1u << 5) | (1u << 6);
 // spring cutting against a blade triangle (sorts the current state first, like the next

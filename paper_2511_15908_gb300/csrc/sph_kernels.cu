@@ -71,6 +71,11 @@ __global__ void __launch_bounds__(kTile, SPH_FORCE_COOP_MINB) k_force_coop(SimCo
 {
     force_coop_item<G>(c, blockIdx.x);
 }
+template <int G>
+__global__ void __launch_bounds__(kTile, SPH_FORCE_COOP_MINB) k_force_ordered(SimConst c)
+{
+    force_ordered_item<G>(c, blockIdx.x);
+}
 __global__ void __launch_bounds__(kTile) k_wrench(SimConst c) { wrench_item(c, blockIdx.x); }
 // the last substep of an update cycle: the cycle's end (the rolling-average log) in the
 // block that finished the wrench, after its sums (the same values k_cycle_end would read)
@@ -163,6 +168,18 @@ int walk_coop(const SimConst &c)
     return c.n <= kCoopAllMax ? 2 : c.n <= kCoopRigidMax && c.n_rigid <= c.n / 8 ? 1 : 0;
 }
 
+static bool force_low_latency(const SimConst &c) { return (c.flags & FLAG_LOW_LATENCY) && !(c.flags & FLAG_VOLUME); }
+static bool force_ordered(const SimConst &c)
+{
+    return c.coop == 2 && c.n <= kForceOrderedMax && !(c.flags & (FLAG_VOLUME | FLAG_LOW_LATENCY));
+}
+int force_blocks(const SimConst &c)
+{
+    const int per = force_low_latency(c) ? kTile / kLowLatencyForceG
+                    : force_ordered(c) ? kTile / kForceOrderedG : kForceThreads;
+    return (c.n + per - 1) / per;
+}
+
 static inline int blocks_for(int n, int t) { return (n + t - 1) / t; }
 
 cudaError_t launch_substep(const SimConst &c, cudaStream_t s, cudaEvent_t *ev, bool external,
@@ -193,7 +210,7 @@ cudaError_t launch_substep(const SimConst &c, cudaStream_t s, cudaEvent_t *ev, b
     // the neighbour search and the sums over its lists (timed together); the volume variant's
     // boundary weights between them.  The low-latency pass's walk has rows for Rc < 2.5 (cells >= h
     // give Rc ~ 2)
-    const bool lanes = (c.flags & FLAG_LOW_LATENCY) && !(c.flags & FLAG_VOLUME) && c.Rc < 2.5f, walk = lanes && c.n <= kLowLatency32Max;
+    const bool lanes = force_low_latency(c) && c.Rc < 2.5f, walk = lanes && c.n <= kLowLatency32Max;
     const auto search = c.coop == 0 ? k_search<0> : c.coop == 1 ? k_search<1> : k_search<2>;
     if (!walk) search<<<search_tiles(c, SPH_SEARCH_THREADS), SPH_SEARCH_THREADS, 0, s>>>(c);
     if (walk) {
@@ -208,9 +225,10 @@ cudaError_t launch_substep(const SimConst &c, cudaStream_t s, cudaEvent_t *ev, b
         density<<<density_tiles(c, SPH_DENSITY_THREADS), SPH_DENSITY_THREADS, 0, s>>>(c);
     }
     mark();
-    // (a flagged scene's n_force_blocks counts blocks of 256 / G particles)
-    if ((c.flags & FLAG_LOW_LATENCY) && !(c.flags & FLAG_VOLUME))
+    if (force_low_latency(c))
         k_force_coop<kLowLatencyForceG><<<c.n_force_blocks, kTile, 0, s>>>(c);
+    else if (force_ordered(c))
+        k_force_ordered<kForceOrderedG><<<c.n_force_blocks, kTile, 0, s>>>(c);
     else if (c.flags & FLAG_VOLUME)
         k_force<true><<<c.n_force_blocks, kForceThreads, 0, s>>>(c);
     else
