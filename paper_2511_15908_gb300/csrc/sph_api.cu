@@ -133,7 +133,7 @@ struct sph_handle {
     bool finalized = false;
     // graphs: 1 and 16 substeps, 1 substep followed by the update cycle's end (the last
     // launch of a call), and the profiling substep with event nodes
-    cudaGraphExec_t exec1 = nullptr, exec16 = nullptr, exec1c = nullptr, exec_prof = nullptr;
+    cudaGraphExec_t exec1 = nullptr, exec16 = nullptr, exec1c = nullptr, exec_haptic = nullptr, exec_prof = nullptr;
     int profiling = 0;                      // 0 off, 1 every kernel, 2 the density pass only
     int prof_graph = 0;                     // the level exec_prof was captured for
     int prof_last = 0;                      // the level of the last profiled substep
@@ -144,7 +144,8 @@ struct sph_handle {
     // 64 on): the copies are truly asynchronous and one stream synchronisation ends a read
     unsigned char *pin = nullptr;
     size_t pin_bytes = 0;
-    char *pin_state = nullptr;           // a small scene's state, in the same memory behind them
+    HapticSlot *slot = nullptr;          // in the same memory, behind them
+    char *pin_state = nullptr;           // and a small scene's state
 };
 
 namespace {
@@ -291,14 +292,14 @@ sph_status finalize(sph_handle *h)
 }
 
 sph_status capture(sph_handle *h, int count, cudaGraphExec_t *out, bool prof = false,
-                   bool cycle_end = false, unsigned ev_mask = ~0u)
+                   bool cycle_end = false, unsigned ev_mask = ~0u, HapticSlot *slot = nullptr)
 {
     cudaGraph_t g = nullptr;
     SPH_CUDA(h, cudaStreamBeginCapture(h->stream, cudaStreamCaptureModeThreadLocal));
     cudaError_t le = cudaSuccess;
     for (int i = 0; i < count && le == cudaSuccess; ++i)
         le = launch_substep(h->c, h->stream, prof ? h->ev : nullptr, prof, cycle_end && i == count - 1,
-                            ev_mask);
+                            ev_mask, slot);
     cudaError_t ce = cudaStreamEndCapture(h->stream, &g);
     if (le != cudaSuccess) { if (g) cudaGraphDestroy(g); return cuda_fail(h, le, "capture launch"); }
     if (ce != cudaSuccess) return cuda_fail(h, ce, "cudaStreamEndCapture");
@@ -454,15 +455,16 @@ sph_status sph_create(const sph_params *p, const sph_capacity *cap, void *d_work
     // pinned staging for the synchronising reads: status, then the counters and the
     // smoothing window's cycle log (host memory; unpinned copies if refused)
     h->pin_bytes = 64 + 16 + 48 * (size_t)c.smooth_window;
-    const size_t pin_end = align256(h->pin_bytes);
+    const size_t slot_end = align256(h->pin_bytes + sizeof(HapticSlot));
     const size_t state_bytes = 256 + 28 * (size_t)cap->max_particles;
     const bool small = state_bytes <= kPinStateMax;
-    if (cudaHostAlloc((void **)&h->pin, pin_end + (small ? kPinStateMax : 0), cudaHostAllocDefault) != cudaSuccess) {
+    if (cudaHostAlloc((void **)&h->pin, slot_end + (small ? kPinStateMax : 0), cudaHostAllocDefault) != cudaSuccess) {
         h->pin = nullptr;
         h->pin_bytes = 0;
         cudaGetLastError();
     } else {
-        if (small) h->pin_state = reinterpret_cast<char *>(h->pin + pin_end);
+        h->slot = reinterpret_cast<HapticSlot *>(h->pin + h->pin_bytes);
+        if (small) h->pin_state = reinterpret_cast<char *>(h->pin + slot_end);
     }
     *out = h;
     return SPH_OK;
@@ -590,14 +592,20 @@ sph_status sph_add_soft(sph_handle *h, int32_t n, const float *h_xyz, float spac
     return SPH_OK;
 }
 
+// may body_id (-1: none) be grabbed?  Finalizes the scene if so
+static sph_status grab_check(sph_handle *h, int32_t body_id)
+{
+    if (body_id >= (int)h->bodies.size() || body_id < -1) return fail(h, SPH_ERR_ARG, "bad body id");
+    if (body_id >= 0 && h->bodies[body_id].kind != SPH_BODY_RIGID)
+        return fail(h, SPH_ERR_ARG, "only rigid bodies can be grabbed");
+    return finalize(h);
+}
+
 sph_status sph_set_grab_pose(sph_handle *h, int32_t body_id, const float pose[7],
                              const float vel[6], const float grab_point_local[3])
 {
     if (!h) return SPH_ERR_ARG;
-    if (body_id >= (int)h->bodies.size() || body_id < -1) return fail(h, SPH_ERR_ARG, "bad body id");
-    if (body_id >= 0 && h->bodies[body_id].kind != SPH_BODY_RIGID)
-        return fail(h, SPH_ERR_ARG, "only rigid bodies can be grabbed");
-    sph_status st = finalize(h);
+    sph_status st = grab_check(h, body_id);
     if (st != SPH_OK) return st;
     float pv[13] = {0, 0, 0, 1, 0, 0, 0, 0, 0, 0, 0, 0, 0};
     float gl[3] = {0, 0, 0};
@@ -943,7 +951,28 @@ sph_status sph_haptic_cycle(sph_handle *h, int32_t body_id, const float pose[7],
                             int32_t n_substeps, int32_t smoothed, double out[6])
 {
     if (!h || !out) return SPH_ERR_ARG;
-    sph_status st = sph_set_grab_pose(h, body_id, pose, vel, nullptr);
+    sph_status st;
+    if (body_id >= 0 && pose && n_substeps == 1 && !smoothed && h->slot && h->stream && !h->profiling &&
+        !(h->p.flags & SPH_FLAG_NO_GRAPH)) {
+        // the haptic tick's form: pose, substep and wrench in one graph launch
+        st = grab_check(h, body_id);
+        if (st != SPH_OK) return st;
+        if (!h->exec_haptic) {
+            st = capture(h, 1, &h->exec_haptic, false, true, ~0u, h->slot);
+            if (st != SPH_OK) return st;
+        }
+        HapticSlot &slot = *h->slot;
+        slot.body = body_id;
+        for (int a = 0; a < 7; ++a) slot.pose_vel[a] = pose[a];
+        for (int a = 0; a < 6; ++a) slot.pose_vel[7 + a] = vel ? vel[a] : 0.0f;
+        SPH_CUDA(h, cudaGraphLaunch(h->exec_haptic, h->stream));
+        h->grab = body_id;
+        h->substeps += 1;
+        SPH_CUDA(h, cudaStreamSynchronize(h->stream));
+        std::memcpy(out, slot.wrench, sizeof slot.wrench);
+        return eval_status(h, slot.status);
+    }
+    st = sph_set_grab_pose(h, body_id, pose, vel, nullptr);
     if (st != SPH_OK) return st;
     st = sph_step(h, n_substeps);
     if (st != SPH_OK) return st;
@@ -1072,6 +1101,7 @@ void sph_destroy(sph_handle *h)
     if (h->exec1) cudaGraphExecDestroy(h->exec1);
     if (h->exec16) cudaGraphExecDestroy(h->exec16);
     if (h->exec1c) cudaGraphExecDestroy(h->exec1c);
+    if (h->exec_haptic) cudaGraphExecDestroy(h->exec_haptic);
     if (h->exec_prof) cudaGraphExecDestroy(h->exec_prof);
     for (int i = 0; i <= kSubstepKernels; ++i)
         if (h->ev[i]) cudaEventDestroy(h->ev[i]);

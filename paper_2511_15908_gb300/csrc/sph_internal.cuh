@@ -114,15 +114,53 @@ struct __align__(16) SimConst {
     uint32_t *ctr;             // [0] substep counter, [1] reduce ticket, [2] cycle counter
 };
 
+// First statement of every kernel of a chain launched with launch_after: lets the next kernel
+// of the chain be put on the GPU beside this one's last blocks, and waits until the kernel
+// before it has finished and its writes can be read.  Nothing of the chain's data may be
+// touched above it.
+__device__ __forceinline__ void chain_enter()
+{
+    asm volatile("griddepcontrol.launch_dependents;");
+    asm volatile("griddepcontrol.wait;" ::: "memory");
+}
+
+// Launches a kernel of a chain (its first statement is chain_enter) so that its blocks take
+// their places while the kernel before it in the stream ends: the launch and the ramp-up of
+// its blocks, ~1-2 us each, then overlap with that kernel's last wave.  A plain launch where
+// early is false.
+template <class... Params, class... Args>
+inline cudaError_t launch_after(bool early, void (*kernel)(Params...), unsigned grid, unsigned threads, size_t smem,
+                                cudaStream_t s, Args &&...args)
+{
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3(grid);
+    cfg.blockDim = dim3(threads);
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = s;
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[0].val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = early ? 1 : 0;
+    return cudaLaunchKernelEx(&cfg, kernel, Params(args)...);
+}
+
 // Launchers (sph_kernels.cu).  All enqueue on `s` and return the launch error.
 constexpr int kSubstepKernels = 8;
 // ev (nullable): kSubstepKernels + 1 events recorded around the kernels; external = record
 // them as graph nodes when the stream is being captured.
 // cycle_end: the update cycle's end (launch_cycle_end's work) folded into the wrench pass;
 // ev_mask: which of the kSubstepKernels + 1 events are recorded (bit k: event k)
+// slot: a haptic cycle's one substep, its pose from there and its wrench to there
+struct HapticSlot {            // in pinned host memory, read and written by the kernels
+    double wrench[6];
+    uint32_t status[3];
+    int body;
+    float pose_vel[13];
+};
 cudaError_t launch_substep(const SimConst &c, cudaStream_t s, cudaEvent_t *ev = nullptr,
                            bool external = false, bool cycle_end = false,
-                           unsigned ev_mask = ~0u);
+                           unsigned ev_mask = ~0u, HapticSlot *slot = nullptr);
 // who walks with cooperating lanes in a scene stepped alone
 int walk_coop(const SimConst &c);
 // blocks (and diagnostic rows) of the force pass of a scene stepped alone

@@ -27,20 +27,45 @@ constexpr int kLowLatency32Max = 20000;
 
 namespace sphgb {
 
-__global__ void __launch_bounds__(kTile) k_hash(SimConst c) { hash_item(c, blockIdx.x); }
-__global__ void __launch_bounds__(kTile) k_scan_tiles(SimConst c) { scan_tiles_item(c, blockIdx.x); }
-__global__ void __launch_bounds__(kTile) k_scan_apply(SimConst c) { scan_apply_item(c, blockIdx.x); }
-__global__ void __launch_bounds__(kTile) k_scan_lookback(SimConst c) { scan_lookback_item(c); }
+__global__ void __launch_bounds__(kTile) k_hash(SimConst c)
+{
+    chain_enter();
+    hash_item(c, blockIdx.x);
+}
+__global__ void __launch_bounds__(kTile) k_scan_tiles(SimConst c)
+{
+    chain_enter();
+    scan_tiles_item(c, blockIdx.x);
+}
+__global__ void __launch_bounds__(kTile) k_scan_apply(SimConst c)
+{
+    chain_enter();
+    scan_apply_item(c, blockIdx.x);
+}
+__global__ void __launch_bounds__(kTile) k_scan_lookback(SimConst c)
+{
+    chain_enter();
+    scan_lookback_item(c);
+}
 // the substep's scan: single-pass (one launch; timed as the tile pass, the apply pass reads
 // ~0) unless built with SPH_SCAN_LOOKBACK=0
 #ifndef SPH_SCAN_LOOKBACK
 #define SPH_SCAN_LOOKBACK 1
 #endif
-__global__ void __launch_bounds__(kTile) k_scatter(SimConst c) { scatter_item(c, blockIdx.x); }
-__global__ void __launch_bounds__(kTile) k_rank_gather(SimConst c) { rank_gather_item(c, blockIdx.x); }
+__global__ void __launch_bounds__(kTile) k_scatter(SimConst c)
+{
+    chain_enter();
+    scatter_item(c, blockIdx.x);
+}
+__global__ void __launch_bounds__(kTile) k_rank_gather(SimConst c)
+{
+    chain_enter();
+    rank_gather_item(c, blockIdx.x);
+}
 template <int COOP, int MODE>
 __global__ void __launch_bounds__(SPH_DENSITY_THREADS, SPH_DENSITY_MINB) k_density(SimConst c)
 {
+    chain_enter();
     density_item<SPH_DENSITY_THREADS, COOP, MODE, true>(c, blockIdx.x);
 }
 #define SPH_SEARCH_THREADS 256
@@ -48,49 +73,61 @@ __global__ void __launch_bounds__(SPH_DENSITY_THREADS, SPH_DENSITY_MINB) k_densi
 template <int COOP>
 __global__ void __launch_bounds__(SPH_SEARCH_THREADS, SPH_SEARCH_MINB) k_search(SimConst c)
 {
+    chain_enter();
     search_item<SPH_SEARCH_THREADS, COOP>(c, blockIdx.x);
 }
 template <int G>
 __global__ void __launch_bounds__(kTile, SPH_LOW_LATENCY_MINB) k_density_walk(SimConst c)
 {
+    chain_enter();
     density_walk_item<G>(c, blockIdx.x);
 }
 template <int G>
 __global__ void __launch_bounds__(kTile, SPH_LOW_LATENCY_MINB) k_density_lanes(SimConst c)
 {
+    chain_enter();
     density_lanes_item<G>(c, blockIdx.x);
 }
-__global__ void __launch_bounds__(kTile) k_boundary_volume(SimConst c) { boundary_volume_item(c, blockIdx.x); }
+__global__ void __launch_bounds__(kTile) k_boundary_volume(SimConst c)
+{
+    chain_enter();
+    boundary_volume_item(c, blockIdx.x);
+}
 template <bool VOL>
 __global__ void __launch_bounds__(kForceThreads, SPH_FORCE_MINB) k_force(SimConst c)
 {
+    chain_enter();
     force_item_v<kForceThreads, VOL>(c, blockIdx.x);
 }
 template <int G>
 __global__ void __launch_bounds__(kTile, SPH_FORCE_COOP_MINB) k_force_coop(SimConst c)
 {
+    chain_enter();
     force_coop_item<G>(c, blockIdx.x);
 }
 template <int G>
 __global__ void __launch_bounds__(kTile, SPH_FORCE_COOP_MINB) k_force_ordered(SimConst c)
 {
+    chain_enter();
     force_ordered_item<G>(c, blockIdx.x);
 }
-__global__ void __launch_bounds__(kTile) k_wrench(SimConst c) { wrench_item(c, blockIdx.x); }
+__global__ void __launch_bounds__(kTile) k_wrench(SimConst c)
+{
+    chain_enter();
+    wrench_item(c, blockIdx.x);
+}
 // the last substep of an update cycle: the cycle's end (the rolling-average log) in the
 // block that finished the wrench, after its sums (the same values k_cycle_end would read)
 __global__ void __launch_bounds__(kTile) k_wrench_cycle(SimConst c)
 {
+    chain_enter();
     if (wrench_item(c, blockIdx.x) && threadIdx.x == 0) cycle_end_item(c);
 }
 __global__ void k_cycle_end(SimConst c) { cycle_end_item(c); }
 
-__global__ void k_set_grab(SimConst c, int body, int grab, float pv0, float pv1, float pv2,
-                           float pv3, float pv4, float pv5, float pv6, float pv7, float pv8,
-                           float pv9, float pv10, float pv11, float pv12, float g0, float g1,
-                           float g2, int set_pose, int path_n)
+__device__ __forceinline__ void set_grab(const SimConst &c, int body, int grab, const float (&pv)[13],
+                                         const float (&gl)[3], int set_pose, int path_n)
 {
-    const float pv[13] = {pv0, pv1, pv2, pv3, pv4, pv5, pv6, pv7, pv8, pv9, pv10, pv11, pv12};
     for (int b = 0; b < c.nb; ++b) {
         DevBody &B = c.body[b];
         if (b != body) {
@@ -99,7 +136,7 @@ __global__ void k_set_grab(SimConst c, int body, int grab, float pv0, float pv1,
         }
         B.grabbed = grab;
         if (!grab) { B.path_n = 0; continue; }
-        B.grab_local[0] = g0; B.grab_local[1] = g1; B.grab_local[2] = g2;
+        for (int a = 0; a < 3; ++a) B.grab_local[a] = gl[a];
         if (set_pose) {
             for (int a = 0; a < 3; ++a) { B.t[a] = pv[a]; B.v[a] = pv[7 + a]; B.w[a] = pv[10 + a]; }
             for (int a = 0; a < 4; ++a) B.q[a] = pv[3 + a];
@@ -107,6 +144,36 @@ __global__ void k_set_grab(SimConst c, int body, int grab, float pv0, float pv1,
         B.path_n = path_n;
         B.path_step0 = (int)c.ctr[0];
     }
+}
+
+__global__ void k_set_grab(SimConst c, int body, int grab, float pv0, float pv1, float pv2,
+                           float pv3, float pv4, float pv5, float pv6, float pv7, float pv8,
+                           float pv9, float pv10, float pv11, float pv12, float g0, float g1,
+                           float g2, int set_pose, int path_n)
+{
+    const float pv[13] = {pv0, pv1, pv2, pv3, pv4, pv5, pv6, pv7, pv8, pv9, pv10, pv11, pv12};
+    const float gl[3] = {g0, g1, g2};
+    set_grab(c, body, grab, pv, gl, set_pose, path_n);
+}
+
+// A haptic cycle's two ends, in its graph: the pose comes from the slot in pinned memory, and the
+// block that finishes the wrench writes it there with the status words.  As launches and copies
+// of their own around the substep's graph the three took some 14 us of a cycle's ~100.
+__global__ void k_haptic_pose(SimConst c, const HapticSlot *slot)
+{
+    chain_enter();
+    float pv[13];
+    for (int a = 0; a < 13; ++a) pv[a] = slot->pose_vel[a];
+    const float gl[3] = {0.0f, 0.0f, 0.0f};
+    set_grab(c, slot->body, 1, pv, gl, 1, 0);
+}
+__global__ void __launch_bounds__(kTile) k_wrench_haptic(SimConst c, HapticSlot *slot)
+{
+    chain_enter();
+    if (!wrench_item(c, blockIdx.x)) return;
+    if (threadIdx.x == 0) cycle_end_item(c);
+    if (threadIdx.x < 6) slot->wrench[threadIdx.x] = c.wrench[6 * slot->body + threadIdx.x];
+    else if (threadIdx.x < 9) slot->status[threadIdx.x - 6] = c.status[threadIdx.x - 6];
 }
 
 // Cell key and id of each sorted slot (test hook): recomputed from the sorted positions.
@@ -183,61 +250,75 @@ int force_blocks(const SimConst &c)
 static inline int blocks_for(int n, int t) { return (n + t - 1) / t; }
 
 cudaError_t launch_substep(const SimConst &c, cudaStream_t s, cudaEvent_t *ev, bool external,
-                           bool cycle_end, unsigned ev_mask)
+                           bool cycle_end, unsigned ev_mask, HapticSlot *slot)
 {
     const int nb = blocks_for(c.n, 256);
+    // The short passes are put on the GPU while the pass before them ends; the long ones start
+    // afterwards: early, their first blocks, the longest, would fill whichever SMs came free first.
+    bool early = s != nullptr;            // (a kernel behind an event waits for the event)
+    cudaError_t err = cudaSuccess;
+    auto go = [&](void (*kernel)(SimConst), unsigned grid, unsigned threads, bool is_short) {
+        if (err == cudaSuccess) err = launch_after(early && is_short, kernel, grid, threads, 0, s, c);
+        early = s != nullptr;
+    };
     int k = 0;
     auto mark = [&]() {
-        if (ev && (ev_mask >> k & 1u)) cudaEventRecordWithFlags(ev[k], s, external ? cudaEventRecordExternal : 0);
+        if (ev && (ev_mask >> k & 1u)) {
+            cudaEventRecordWithFlags(ev[k], s, external ? cudaEventRecordExternal : 0);
+            early = false;
+        }
         ++k;
     };
+    if (slot) err = launch_after(false, k_haptic_pose, 1, 1, 0, s, c, slot);
     mark();
-    k_hash<<<nb, kTile, 0, s>>>(c);
+    go(k_hash, nb, kTile, true);
     mark();
     if (SPH_SCAN_LOOKBACK) {
-        k_scan_lookback<<<c.n_scan_tiles, kTile, 0, s>>>(c);
+        go(k_scan_lookback, c.n_scan_tiles, kTile, true);
         mark();
     } else {
-        k_scan_tiles<<<c.n_scan_tiles, kTile, 0, s>>>(c);
+        go(k_scan_tiles, c.n_scan_tiles, kTile, true);
         mark();
-        k_scan_apply<<<c.n_scan_tiles, kTile, 0, s>>>(c);
+        go(k_scan_apply, c.n_scan_tiles, kTile, true);
     }
     mark();
-    k_scatter<<<nb, kTile, 0, s>>>(c);
+    go(k_scatter, nb, kTile, true);
     mark();
-    k_rank_gather<<<nb, kTile, 0, s>>>(c);
+    go(k_rank_gather, nb, kTile, true);
     mark();
     // the neighbour search and the sums over its lists (timed together); the volume variant's
     // boundary weights between them.  The low-latency pass's walk has rows for Rc < 2.5 (cells >= h
     // give Rc ~ 2)
     const bool lanes = force_low_latency(c) && c.Rc < 2.5f, walk = lanes && c.n <= kLowLatency32Max;
     const auto search = c.coop == 0 ? k_search<0> : c.coop == 1 ? k_search<1> : k_search<2>;
-    if (!walk) search<<<search_tiles(c, SPH_SEARCH_THREADS), SPH_SEARCH_THREADS, 0, s>>>(c);
+    if (!walk) go(search, search_tiles(c, SPH_SEARCH_THREADS), SPH_SEARCH_THREADS, false);
     if (walk) {
-        k_density_walk<32><<<(unsigned)tiles_of<32>(c.n, kTile), kTile, 0, s>>>(c);
+        go(k_density_walk<32>, (unsigned)tiles_of<32>(c.n, kTile), kTile, false);
     } else if (lanes) {
-        k_density_lanes<16><<<(unsigned)tiles_of<16>(c.n, kTile), kTile, 0, s>>>(c);
+        go(k_density_lanes<16>, (unsigned)tiles_of<16>(c.n, kTile), kTile, false);
     } else {
         const bool vol = (c.flags & FLAG_VOLUME) != 0;
-        if (vol && c.n > c.nf) k_boundary_volume<<<blocks_for(c.n - c.nf, kTile), kTile, 0, s>>>(c);
+        if (vol && c.n > c.nf) go(k_boundary_volume, blocks_for(c.n - c.nf, kTile), kTile, false);
         const auto density = vol ? (c.coop == 0 ? k_density<0, DENSITY_VOLUME> : c.coop == 1 ? k_density<1, DENSITY_VOLUME> : k_density<2, DENSITY_VOLUME>)
                                  : (c.coop == 0 ? k_density<0, DENSITY_MASS> : c.coop == 1 ? k_density<1, DENSITY_MASS> : k_density<2, DENSITY_MASS>);
-        density<<<density_tiles(c, SPH_DENSITY_THREADS), SPH_DENSITY_THREADS, 0, s>>>(c);
+        go(density, density_tiles(c, SPH_DENSITY_THREADS), SPH_DENSITY_THREADS, false);
     }
     mark();
     if (force_low_latency(c))
-        k_force_coop<kLowLatencyForceG><<<c.n_force_blocks, kTile, 0, s>>>(c);
+        go(k_force_coop<kLowLatencyForceG>, c.n_force_blocks, kTile, false);
     else if (force_ordered(c))
-        k_force_ordered<kForceOrderedG><<<c.n_force_blocks, kTile, 0, s>>>(c);
+        go(k_force_ordered<kForceOrderedG>, c.n_force_blocks, kTile, false);
     else if (c.flags & FLAG_VOLUME)
-        k_force<true><<<c.n_force_blocks, kForceThreads, 0, s>>>(c);
+        go(k_force<true>, c.n_force_blocks, kForceThreads, false);
     else
-        k_force<false><<<c.n_force_blocks, kForceThreads, 0, s>>>(c);
+        go(k_force<false>, c.n_force_blocks, kForceThreads, false);
     mark();
-    if (cycle_end) k_wrench_cycle<<<c.n_wgrid, kTile, 0, s>>>(c);
-    else k_wrench<<<c.n_wgrid, kTile, 0, s>>>(c);
+    if (slot && err == cudaSuccess) err = launch_after(early, k_wrench_haptic, c.n_wgrid, kTile, 0, s, c, slot);
+    else if (cycle_end) go(k_wrench_cycle, c.n_wgrid, kTile, true);
+    else go(k_wrench, c.n_wgrid, kTile, true);
     mark();
-    return cudaGetLastError();
+    const cudaError_t last = cudaGetLastError();
+    return err != cudaSuccess ? err : last;
 }
 
 __global__ void __launch_bounds__(kTile) k_cut(SimConst c, Blade t, unsigned *count)

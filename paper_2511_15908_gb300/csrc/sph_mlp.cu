@@ -155,6 +155,7 @@ __global__ void k_train_update(GradSrc src, float *w, float *m, float *v, float 
                                float eps, float c1, float c2, Images im, const double *loss_part, int nblk, int B,
                                double *loss)
 {
+    chain_enter();
     const int t = blockIdx.x * blockDim.x + threadIdx.x;
     if (t == 0) finish_loss(loss_part, nblk, B, loss);
     if (t >= kParams) return;
@@ -589,6 +590,7 @@ __global__ void __launch_bounds__(kMlpThreads, 1) k_mlp(const __grid_constant__ 
         for (int c = 0; c < chunks; ++c) tma_load_2d(dst + (uint32_t)c * stride, &maps.m[l], c * kTcKChunk, 0, full(l));
         loading |= 1u << l;
     };
+    chain_enter();
     if (tid == 0) {
         for (int l = 0; l < 8; ++l) mbar_init(full(l));
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
@@ -946,8 +948,8 @@ sph_status mlp_launch(sph_mlp *m, const MlpArgs &a)
     if (!m->mapped) return mfail(m, SPH_ERR_CUDA, "the weights' tensor maps could not be built");
     static std::atomic<unsigned long long> configured{0};
     MLP_CUDA(m, smem_opt_in(k_mlp<TRAIN>, kMlpSmem, configured));
-    k_mlp<TRAIN><<<(a.B + kTcM - 1) / kTcM, kMlpThreads, kMlpSmem, m->stream>>>(m->maps, a);
-    MLP_CUDA(m, cudaGetLastError());
+    MLP_CUDA(m, launch_after(m->stream != nullptr, k_mlp<TRAIN>, (a.B + kTcM - 1) / kTcM, kMlpThreads, kMlpSmem, m->stream,
+                             m->maps, a));
     return SPH_OK;
 }
 
@@ -1126,10 +1128,8 @@ sph_status sph_mlp_train_step(sph_mlp *m, const float *d_x, const float *d_t, in
     const float c1 = 1.0f / (1.0f - std::pow(b1, (float)m->adam_t));
     const float c2 = 1.0f / (1.0f - std::pow(b2, (float)m->adam_t));
     const Images im{m->w1b, m->w2b, m->w3b, m->w4b, m->w2t, m->w3t, m->w4t, m->b4pad};
-    k_train_update<<<(kParams + 255) / 256, 256, 0, m->stream>>>(src, m->master, m->m, m->v, m->grad, lr, b1, b2,
-                                                                 1e-8f, c1, c2, im, m->loss_part, nblk, batch,
-                                                                 m->loss);
-    MLP_CUDA(m, cudaGetLastError());
+    MLP_CUDA(m, launch_after(m->stream != nullptr, k_train_update, (kParams + 255) / 256, 256, 0, m->stream, src, m->master,
+                             m->m, m->v, m->grad, lr, b1, b2, 1e-8f, c1, c2, im, m->loss_part, nblk, batch, m->loss));
     if (h_loss) {
         MLP_CUDA(m, cudaMemcpyAsync(h_loss, m->loss, 8, cudaMemcpyDeviceToHost, m->stream));
         return mlp_status(m);

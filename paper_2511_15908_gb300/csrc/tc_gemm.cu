@@ -34,6 +34,7 @@ __global__ void __launch_bounds__(kTcThreads, 1) k_tc_gemm(const __grid_constant
     extern __shared__ unsigned char smem_raw[];
     __shared__ uint32_t s_tmem;
     __shared__ int s_fail;
+    chain_enter();
     int w = 0;
     while (w + 1 < group.count && (int)blockIdx.x >= group.first[w + 1]) ++w;
     const TcGemm &g = group.g[w];
@@ -222,8 +223,7 @@ cudaError_t tc_gemm_group(const TcGemm *g, int count, unsigned *status, cudaStre
         const int ct = (q.N + grp.ntile[i] - 1) / grp.ntile[i];
         grp.first[i + 1] = grp.first[i] + (q.M + kTcM - 1) / kTcM * ct * q.ksplit;
     }
-    k_tc_gemm<<<grp.first[count], kTcThreads, kSmemBytes, s>>>(grp);
-    return cudaGetLastError();
+    return launch_after(s != nullptr, k_tc_gemm, grp.first[count], kTcThreads, kSmemBytes, s, grp);
 }
 
 }  // namespace sphgb

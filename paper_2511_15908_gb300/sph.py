@@ -176,7 +176,7 @@ def load(path: str = LIB_PATH):
     L.sph_surrogate_anchor.restype = st
     L.sph_surrogate_anchor.argtypes = [_vp, _vp]
     L.sph_surrogate_tick.restype = st
-    L.sph_surrogate_tick.argtypes = [_vp, _f32p, ctypes.c_float, _f64p]
+    L.sph_surrogate_tick.argtypes = [_vp, _vp, ctypes.c_float, _vp]
     L.sph_surrogate_features.restype = st
     L.sph_surrogate_features.argtypes = [_vp, _vp, ctypes.c_int32, _vp, ctypes.c_int32, _vp, ctypes.c_int32, _vp]
     L.sph_surrogate_targets.restype = st
@@ -185,8 +185,7 @@ def load(path: str = LIB_PATH):
     L.sph_measure_fp32_fma.argtypes = [_vp, ctypes.c_int32, ctypes.c_int32, _vp,
                                        ctypes.POINTER(ctypes.c_double)]
     L.sph_haptic_cycle.restype = st
-    L.sph_haptic_cycle.argtypes = [_vp, ctypes.c_int32, _f32p, _f32p, ctypes.c_int32, ctypes.c_int32,
-                                   ctypes.POINTER(ctypes.c_double)]
+    L.sph_haptic_cycle.argtypes = [_vp, ctypes.c_int32, _vp, _vp, ctypes.c_int32, ctypes.c_int32, _vp]
     L.sph_checkpoint_bytes.restype = ctypes.c_size_t
     L.sph_checkpoint_bytes.argtypes = [_vp]
     L.sph_checkpoint_save.restype = st
@@ -358,8 +357,8 @@ class Simulation:
         vel = np.ascontiguousarray(vel, np.float32)
         if out is None:
             out = np.zeros(6, np.float64)
-        self._check(self.L.sph_haptic_cycle(self.h, body, _ptr(pose, ctypes.c_float), _ptr(vel, ctypes.c_float),
-                                            int(n_substeps), int(smoothed), _ptr(out, ctypes.c_double)))
+        self._check(self.L.sph_haptic_cycle(self.h, body, pose.ctypes.data, vel.ctypes.data, int(n_substeps),
+                                            int(smoothed), out.ctypes.data))
         return out
 
     def set_grab_path(self, path):
@@ -653,8 +652,7 @@ class Surrogate:
         """Wrench at a haptic tick: anchor wrench + predicted change (host, 6 doubles)."""
         pv = np.ascontiguousarray(pose_vel, np.float32)
         out = np.zeros(6, np.float64) if out is None else out
-        self._check(self.L.sph_surrogate_tick(self.m, _ptr(pv, ctypes.c_float), float(elapsed),
-                                              _ptr(out, ctypes.c_double)))
+        self._check(self.L.sph_surrogate_tick(self.m, pv.ctypes.data, float(elapsed), out.ctypes.data))
         return out
 
     def features(self, ticks_dev, anchors_dev, elapsed_dev):
