@@ -28,7 +28,10 @@ struct BatchConst {
     int n_scenes;
     int chunk;                    // tiles per queue fetch
     int total[kPhases];           // tiles of each phase over all scenes
-    const int *prefix;            // kPhases x (n_scenes + 1) tile prefix per phase
+    int rigid;                    // of the density phase's: the rigid particles' tiles, which are the
+                                  // longest and come first, before any scene's others
+    const int *prefix;            // (kPhases + 1) x (n_scenes + 1) tile prefix per phase; the
+                                  // density phase's without the rigid tiles, those in the last row
     const SimConst *scenes;
     unsigned *queue;              // kPhases work-queue counters
     unsigned *bar;                // [0] arrivals, [1] generation
@@ -72,14 +75,27 @@ __device__ bool grid_barrier(const BatchConst &b)
     return s_ok != 0;
 }
 
-__device__ __forceinline__ int scene_of(const int *prefix, int n, int item)
+// The scene whose tile `it` of phase ph is, and the tile's number in it (of the density phase:
+// among the scene's rigid tiles, or, with `rest`, among the others).  All threads of the block
+// compare one prefix each: a binary search is a chain of log2(scenes) loads, ~0.6 us each, before
+// every tile.
+struct BatchTile {
+    int scene, blk;
+    bool rest;
+};
+__device__ __forceinline__ BatchTile batch_tile(const BatchConst &b, int ph, int it)
 {
-    int lo = 0, hi = n;                       // prefix[lo] <= item < prefix[hi]
-    while (hi - lo > 1) {
-        int mid = (lo + hi) >> 1;
-        if (prefix[mid] <= item) lo = mid; else hi = mid;
+    BatchTile t;
+    t.rest = ph == P_DENSITY && it >= b.rigid;
+    if (t.rest) it -= b.rigid;
+    const int *pre = b.prefix + (ph == P_DENSITY && !t.rest ? (int)kPhases : ph) * (b.n_scenes + 1);
+    t.scene = 0;                              // scenes that end at or before the tile
+    for (int i0 = 0; i0 < b.n_scenes; i0 += kTile) {
+        const int i = i0 + (int)threadIdx.x;
+        t.scene += __syncthreads_count(i < b.n_scenes && pre[i + 1] <= it);
     }
-    return lo;
+    t.blk = it - pre[t.scene];
+    return t;
 }
 
 #ifndef SPH_BATCH_MINB
@@ -97,7 +113,6 @@ __global__ void __launch_bounds__(kTile, SPH_BATCH_MINB) k_batch(BatchConst b, i
     int staged = -1;                  // the scene whose constants s_c holds (block-uniform)
     for (int sub = 0; sub < n_substeps; ++sub) {
         for (int ph = 0; ph < kPhases; ++ph) {
-            const int *pre = b.prefix + ph * (b.n_scenes + 1);
             for (;;) {
                 if (threadIdx.x == 0) s_item = (int)atomicAdd(b.queue + ph, (unsigned)b.chunk);
                 __syncthreads();
@@ -106,8 +121,8 @@ __global__ void __launch_bounds__(kTile, SPH_BATCH_MINB) k_batch(BatchConst b, i
                 if (base >= b.total[ph]) break;
                 const int end = min(base + b.chunk, b.total[ph]);
                 for (int it = base; it < end; ++it) {
-                    const int s = scene_of(pre, b.n_scenes, it);
-                    const int blk = it - pre[s];
+                    const BatchTile t = batch_tile(b, ph, it);
+                    const int s = t.scene;
                     // consecutive tiles mostly belong to one scene: stage its constants only
                     // when the scene changes (a substep's counter lives in global memory,
                     // so the staged copy stays valid across phases and substeps)
@@ -120,6 +135,7 @@ __global__ void __launch_bounds__(kTile, SPH_BATCH_MINB) k_batch(BatchConst b, i
                     }
                     __syncthreads();
                     const SimConst &c = s_c;
+                    const int blk = t.blk + (t.rest ? rigid_tiles(c, kTile) : 0);
                     switch (ph) {
                     case P_HASH: hash_item(c, blk); break;
                     case P_SCAN_T: scan_tiles_item(c, blk); break;
@@ -160,17 +176,15 @@ template <int PH>
 __global__ void __launch_bounds__(kTile, batch_phase_minb<PH>()) k_batch_phase(BatchConst b)
 {
     __shared__ __align__(16) SimConst s_c;
-    const int *pre = b.prefix + PH * (b.n_scenes + 1);
-    const int it = blockIdx.x;
-    const int s = scene_of(pre, b.n_scenes, it);
-    const int blk = it - pre[s];
+    const BatchTile t = batch_tile(b, PH, blockIdx.x);
     {
-        const int4 *src = reinterpret_cast<const int4 *>(b.scenes + s);
+        const int4 *src = reinterpret_cast<const int4 *>(b.scenes + t.scene);
         int4 *dst = reinterpret_cast<int4 *>(&s_c);
         for (int w = threadIdx.x; w < (int)(sizeof(SimConst) / 16); w += kTile) dst[w] = __ldg(src + w);
     }
     __syncthreads();
     const SimConst &c = s_c;
+    const int blk = t.blk + (t.rest ? rigid_tiles(c, kTile) : 0);
     switch (PH) {
     case P_HASH: hash_item(c, blk); break;
     case P_SCAN_T: scan_tiles_item(c, blk); break;
@@ -242,7 +256,7 @@ BatchLayout batch_layout(int n)
     size_t off = 0;
     auto take = [&](size_t bytes) { size_t r = off; off = a256(off + bytes); return r; };
     L.scenes = take(sizeof(SimConst) * (size_t)n);
-    L.prefix = take(4 * (size_t)kPhases * (n + 1));
+    L.prefix = take(4 * (size_t)(kPhases + 1) * (n + 1));
     L.queue = take(4 * kPhases);
     L.bar = take(8);
     L.status = take(4);
@@ -432,8 +446,8 @@ sph_status sph_batch_create(sph_handle *const *scenes, int32_t n_scenes, void *d
     bc.n_scenes = n_scenes;
     bc.chunk = 1;
     bc.spin_limit = kBarrierSpin;
-    std::vector<int> prefix((size_t)kPhases * (n_scenes + 1), 0);
-    for (int ph = 0; ph < kPhases; ++ph) {
+    std::vector<int> prefix((size_t)(kPhases + 1) * (n_scenes + 1), 0);
+    for (int ph = 0; ph <= kPhases; ++ph) {          // (the last: the density phase's rigid tiles)
         int run = 0;
         for (int s = 0; s < n_scenes; ++s) {
             prefix[(size_t)ph * (n_scenes + 1) + s] = run;
@@ -442,13 +456,16 @@ sph_status sph_batch_create(sph_handle *const *scenes, int32_t n_scenes, void *d
                         : (ph == P_WRENCH) ? c.n_wgrid
                         : (ph == P_VOLUME) ? ((c.flags & FLAG_VOLUME) ? (c.n - c.nf + kTile - 1) / kTile : 0)
                         : (ph == P_SEARCH) ? search_tiles(c, kTile)
-                        : (ph == P_DENSITY) ? density_tiles(c, kTile)
+                        : (ph == P_DENSITY) ? slot_tiles(c, kTile)
+                        : (ph == kPhases) ? rigid_tiles(c, kTile)
                         : (c.n + kTile - 1) / kTile;
             run += tiles;
         }
         prefix[(size_t)ph * (n_scenes + 1) + n_scenes] = run;
-        bc.total[ph] = run;
+        if (ph < kPhases) bc.total[ph] = run;
+        else bc.rigid = run;
     }
+    bc.total[P_DENSITY] += bc.rigid;
     bc.scenes = (const SimConst *)(b->ws + L.scenes);
     bc.prefix = (const int *)(b->ws + L.prefix);
     bc.queue = (unsigned *)(b->ws + L.queue);
