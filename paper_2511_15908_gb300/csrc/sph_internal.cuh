@@ -15,8 +15,8 @@ constexpr int kMaxBodies = 64;
 constexpr int kMaxCellRun = 1536;   // particles scanned per x-run of cells before the
                                     // status word reports SPH_ERR_CAPACITY
 constexpr int kMaxCell = 512;       // particles per cell for the deterministic rank
-// Lanes per particle of the low-latency force pass (SPH_FLAG_LOW_LATENCY): its grid has
-// this many blocks for each 256 particles, and as many diagnostic rows.
+// Shares per particle of the low-latency force pass (SPH_FLAG_LOW_LATENCY), one or two to a lane:
+// its grid has at most this many blocks for each 256 particles, and as many diagnostic rows.
 #ifndef SPH_LOW_LATENCY_FORCE_G
 #define SPH_LOW_LATENCY_FORCE_G 8
 #endif

@@ -106,6 +106,12 @@ __global__ void __launch_bounds__(kTile, SPH_FORCE_COOP_MINB) k_force_coop(SimCo
     force_coop_item<G>(c, blockIdx.x);
 }
 template <int G>
+__global__ void __launch_bounds__(kTile, SPH_FORCE_COOP_MINB) k_force_shares(SimConst c)
+{
+    chain_enter();
+    force_shares_item<G>(c, blockIdx.x);
+}
+template <int G>
 __global__ void __launch_bounds__(kTile, SPH_FORCE_COOP_MINB) k_force_ordered(SimConst c)
 {
     chain_enter();
@@ -242,7 +248,7 @@ static bool force_ordered(const SimConst &c)
 }
 int force_blocks(const SimConst &c)
 {
-    const int per = force_low_latency(c) ? kTile / kLowLatencyForceG
+    const int per = force_low_latency(c) ? (c.n <= kLowLatency32Max ? 1 : 2) * kTile / kLowLatencyForceG
                     : force_ordered(c) ? kTile / kForceOrderedG : kForceThreads;
     return (c.n + per - 1) / per;
 }
@@ -305,7 +311,8 @@ cudaError_t launch_substep(const SimConst &c, cudaStream_t s, cudaEvent_t *ev, b
     }
     mark();
     if (force_low_latency(c))
-        go(k_force_coop<kLowLatencyForceG>, c.n_force_blocks, kTile, false);
+        go(c.n <= kLowLatency32Max ? k_force_coop<kLowLatencyForceG> : k_force_shares<kLowLatencyForceG>,
+           c.n_force_blocks, kTile, false);
     else if (force_ordered(c))
         go(k_force_ordered<kForceOrderedG>, c.n_force_blocks, kTile, false);
     else if (c.flags & FLAG_VOLUME)
