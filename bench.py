@@ -361,7 +361,7 @@ def batched_set(name, make, args, cells=(1.001, 2.002)):
            "autotuned": {"cell_over_h": cell, "blocks_per_sm": bps, "tiles_per_fetch": info["tiles_per_fetch"],
                          "sms": info["sms"], "candidates": trials},
            "grab_wrench_rel_diff_vs_one_by_one": werr,
-           "gpu_launches_per_step": (9 if bps == 0 else 8 * len(scs) if bps < 0 else 1),
+           "gpu_launches_per_step": (10 if bps == 0 else 8 * len(scs) if bps < 0 else 1),
            "launch_structure": ("one kernel per phase over all scenes" if bps == 0
                                 else "every scene's own kernels as branches of one graph" if bps < 0
                                 else "one persistent cooperative kernel"),
@@ -870,10 +870,10 @@ def run_ours(args):
                                      "settled fill",
                            "out_of_domain_reports": domain[0],
                            "density_pass": ("low latency: 32 or 16 threads per particle"
-                                            if args.low_latency else "one thread per particle")},
-                # per timed substep: hash, single-pass scan, scatter, rank + gather, density,
-                # force, wrench, cycle end
-                "gpu_launches": 8 * args.steps,
+                                            if args.low_latency else "neighbour search, then sums over its lists")},
+                # per timed substep: hash, single-pass scan, scatter, rank + gather, search, density
+                # sums, force, wrench, cycle end
+                "gpu_launches": 9 * args.steps,
                 "kernel_ms": {k: float(v) for k, v in zip(sph.KERNELS, kmean)},
                 "kernel_share": shares,
                 "kernel_ms_source": "a pass of the same substeps after the timed region, events "
@@ -889,10 +889,10 @@ def run_ours(args):
                                 "achieved_gbs": density_hbm, "frac": density_hbm / peaks["hbm_gbs"]},
                 "grab_wrench_err_vs_oracle": wrench_err,
                 "acc_parity": acc_parity,
-                "e2e": {"value": e2e_value, "unit": UNIT, "h2d_bytes_per_step": 64,
+                "e2e": {"value": e2e_value, "unit": UNIT, "h2d_bytes_per_step": 56,
                         "d2h_bytes_per_step": 60,
-                        "what": "sph_haptic_cycle: host pose and velocity in (as kernel "
-                                "arguments), one substep, host wrench out (synchronising); "
+                        "what": "sph_haptic_cycle: host pose and velocity in (through pinned "
+                                "memory), one substep, host wrench out (synchronising); "
                                 "per-kernel profiling off, as in a user's haptic loop"},
                 "clocks": clk.summary(),
                 "cpu_baseline": cpu,
