@@ -361,7 +361,7 @@ def batched_set(name, make, args, cells=(1.001, 2.002)):
            "autotuned": {"cell_over_h": cell, "blocks_per_sm": bps, "tiles_per_fetch": info["tiles_per_fetch"],
                          "sms": info["sms"], "candidates": trials},
            "grab_wrench_rel_diff_vs_one_by_one": werr,
-           "gpu_launches_per_step": (10 if bps == 0 else 8 * len(scs) if bps < 0 else 1),
+           "gpu_launches_per_step": (9 if bps == 0 else 8 * len(scs) if bps < 0 else 1),
            "launch_structure": ("one kernel per phase over all scenes" if bps == 0
                                 else "every scene's own kernels as branches of one graph" if bps < 0
                                 else "one persistent cooperative kernel"),

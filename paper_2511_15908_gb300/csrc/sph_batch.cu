@@ -19,7 +19,7 @@
 
 namespace sphgb {
 
-enum Phase { P_HASH, P_SCAN_T, P_SCAN_A, P_SCATTER, P_GATHER, P_SEARCH, P_VOLUME, P_DENSITY, P_FORCE, P_WRENCH,
+enum Phase { P_HASH, P_SCAN, P_SCATTER, P_GATHER, P_SEARCH, P_VOLUME, P_DENSITY, P_FORCE, P_WRENCH,
              kPhases };
 
 constexpr unsigned kBarrierSpin = 1u << 22;   // x 64 ns sleep: the barrier gives up after ~0.3 s
@@ -138,16 +138,15 @@ __global__ void __launch_bounds__(kTile, SPH_BATCH_MINB) k_batch(BatchConst b, i
                     const int blk = t.blk + (t.rest ? rigid_tiles(c, kTile) : 0);
                     switch (ph) {
                     case P_HASH: hash_item(c, blk); break;
-                    case P_SCAN_T: scan_tiles_item(c, blk); break;
-                    case P_SCAN_A: scan_apply_item(c, blk); break;
+                    case P_SCAN: scan_lookback_item(c); break;
                     case P_SCATTER: scatter_item(c, blk); break;
                     case P_GATHER: rank_gather_item(c, blk); break;
                     case P_SEARCH: search_item<kTile, 0>(c, blk); break;
                     case P_VOLUME: boundary_volume_item(c, blk); break;
                     case P_DENSITY:
-        if (c.flags & FLAG_VOLUME) density_item<kTile, 0, DENSITY_VOLUME, false>(c, blk);
-        else density_item<kTile, 0, DENSITY_MASS, false>(c, blk);
-        break;
+                        if (c.flags & FLAG_VOLUME) density_item<kTile, 0, DENSITY_VOLUME, false>(c, blk);
+                        else density_item<kTile, 0, DENSITY_MASS, false>(c, blk);
+                        break;
                     case P_FORCE: force_item(c, blk); break;
                     default: wrench_item(c, blk); break;
                     }
@@ -187,8 +186,7 @@ __global__ void __launch_bounds__(kTile, batch_phase_minb<PH>()) k_batch_phase(B
     const int blk = t.blk + (t.rest ? rigid_tiles(c, kTile) : 0);
     switch (PH) {
     case P_HASH: hash_item(c, blk); break;
-    case P_SCAN_T: scan_tiles_item(c, blk); break;
-    case P_SCAN_A: scan_apply_item(c, blk); break;
+    case P_SCAN: scan_lookback_item(c); break;
     case P_SCATTER: scatter_item(c, blk); break;
     case P_GATHER: rank_gather_item(c, blk); break;
     case P_SEARCH: search_item<kTile, 0>(c, blk); break;
@@ -282,8 +280,7 @@ cudaError_t launch_phases(sph_batch *b, int n_substeps, int cycle_end)
     const BatchConst &bc = b->bc;
     for (int i = 0; i < n_substeps; ++i) {
         if (bc.total[P_HASH]) k_batch_phase<P_HASH><<<bc.total[P_HASH], kTile, 0, b->stream>>>(bc);
-        if (bc.total[P_SCAN_T]) k_batch_phase<P_SCAN_T><<<bc.total[P_SCAN_T], kTile, 0, b->stream>>>(bc);
-        if (bc.total[P_SCAN_A]) k_batch_phase<P_SCAN_A><<<bc.total[P_SCAN_A], kTile, 0, b->stream>>>(bc);
+        if (bc.total[P_SCAN]) k_batch_phase<P_SCAN><<<bc.total[P_SCAN], kTile, 0, b->stream>>>(bc);
         if (bc.total[P_SCATTER]) k_batch_phase<P_SCATTER><<<bc.total[P_SCATTER], kTile, 0, b->stream>>>(bc);
         if (bc.total[P_GATHER]) k_batch_phase<P_GATHER><<<bc.total[P_GATHER], kTile, 0, b->stream>>>(bc);
         if (bc.total[P_SEARCH]) k_batch_phase<P_SEARCH><<<bc.total[P_SEARCH], kTile, 0, b->stream>>>(bc);
@@ -452,7 +449,7 @@ sph_status sph_batch_create(sph_handle *const *scenes, int32_t n_scenes, void *d
         for (int s = 0; s < n_scenes; ++s) {
             prefix[(size_t)ph * (n_scenes + 1) + s] = run;
             const SimConst &c = table[s];
-            int tiles = (ph == P_SCAN_T || ph == P_SCAN_A) ? c.n_scan_tiles
+            int tiles = (ph == P_SCAN) ? c.n_scan_tiles
                         : (ph == P_WRENCH) ? c.n_wgrid
                         : (ph == P_VOLUME) ? ((c.flags & FLAG_VOLUME) ? (c.n - c.nf + kTile - 1) / kTile : 0)
                         : (ph == P_SEARCH) ? search_tiles(c, kTile)
