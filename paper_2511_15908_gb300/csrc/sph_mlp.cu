@@ -948,8 +948,9 @@ sph_status mlp_launch(sph_mlp *m, const MlpArgs &a)
     if (!m->mapped) return mfail(m, SPH_ERR_CUDA, "the weights' tensor maps could not be built");
     static std::atomic<unsigned long long> configured{0};
     MLP_CUDA(m, smem_opt_in(k_mlp<TRAIN>, kMlpSmem, configured));
-    MLP_CUDA(m, launch_after(m->stream != nullptr, k_mlp<TRAIN>, (a.B + kTcM - 1) / kTcM, kMlpThreads, kMlpSmem, m->stream,
-                             m->maps, a));
+    // (a plain launch: it reads the weights through the read-only path, behind the update's writes)
+    k_mlp<TRAIN><<<(a.B + kTcM - 1) / kTcM, kMlpThreads, kMlpSmem, m->stream>>>(m->maps, a);
+    MLP_CUDA(m, cudaGetLastError());
     return SPH_OK;
 }
 
