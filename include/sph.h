@@ -149,8 +149,8 @@ typedef struct {
 
 /* Bytes of device workspace a scene with these parameters and capacities needs
  * (0 if the arguments are invalid).  The grid size follows from domain and cell; with
- * SPH_FLAG_LOW_LATENCY the force pass's diagnostic rows take 8 times their usual
- * 256 bytes per 1,024 particles (so the flag is part of the parameters the size is
+ * SPH_FLAG_LOW_LATENCY the force pass's diagnostic rows take up to 4 times their usual
+ * 512 bytes per 1,024 particles (so the flag is part of the parameters the size is
  * computed for). */
 size_t sph_workspace_bytes(const sph_params *p, const sph_capacity *cap);
 
