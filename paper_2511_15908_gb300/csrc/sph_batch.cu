@@ -141,13 +141,13 @@ __global__ void __launch_bounds__(kTile, SPH_BATCH_MINB) k_batch(BatchConst b, i
                     case P_SCAN: scan_lookback_item(c); break;
                     case P_SCATTER: scatter_item(c, blk); break;
                     case P_GATHER: rank_gather_item(c, blk); break;
-                    case P_SEARCH: search_item<kTile, 0>(c, blk); break;
-                    case P_VOLUME: boundary_volume_item(c, blk); break;
+                    case P_SEARCH: search_item<kTile, 0, Coherent>(c, blk); break;
+                    case P_VOLUME: boundary_volume_item<Coherent>(c, blk); break;
                     case P_DENSITY:
-                        if (c.flags & FLAG_VOLUME) density_item<kTile, 0, DENSITY_VOLUME, false>(c, blk);
-                        else density_item<kTile, 0, DENSITY_MASS, false>(c, blk);
+                        if (c.flags & FLAG_VOLUME) density_item<kTile, 0, DENSITY_VOLUME, false, Coherent>(c, blk);
+                        else density_item<kTile, 0, DENSITY_MASS, false, Coherent>(c, blk);
                         break;
-                    case P_FORCE: force_item(c, blk); break;
+                    case P_FORCE: force_item<Coherent>(c, blk); break;
                     default: wrench_item(c, blk); break;
                     }
                     __syncthreads();
@@ -189,13 +189,13 @@ __global__ void __launch_bounds__(kTile, batch_phase_minb<PH>()) k_batch_phase(B
     case P_SCAN: scan_lookback_item(c); break;
     case P_SCATTER: scatter_item(c, blk); break;
     case P_GATHER: rank_gather_item(c, blk); break;
-    case P_SEARCH: search_item<kTile, 0>(c, blk); break;
-    case P_VOLUME: boundary_volume_item(c, blk); break;
+    case P_SEARCH: search_item<kTile, 0, ReadOnly>(c, blk); break;
+    case P_VOLUME: boundary_volume_item<ReadOnly>(c, blk); break;
     case P_DENSITY:
-        if (c.flags & FLAG_VOLUME) density_item<kTile, 0, DENSITY_VOLUME, false>(c, blk);
-        else density_item<kTile, 0, DENSITY_MASS, false>(c, blk);
+        if (c.flags & FLAG_VOLUME) density_item<kTile, 0, DENSITY_VOLUME, false, ReadOnly>(c, blk);
+        else density_item<kTile, 0, DENSITY_MASS, false, ReadOnly>(c, blk);
         break;
-    case P_FORCE: force_item(c, blk); break;
+    case P_FORCE: force_item<ReadOnly>(c, blk); break;
     default: wrench_item(c, blk); break;
     }
 }

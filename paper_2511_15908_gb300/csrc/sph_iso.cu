@@ -222,7 +222,7 @@ __global__ void __launch_bounds__(kTile) k_iso_field(SimConst c, IsoGrid g, floa
     const float *vw = reinterpret_cast<const float *>(c.vA) + 3;   // id bits, stride 4
     DensitySum acc;
     uint32_t bad = 0;
-    for_each_row(c, p, bad, [&](int s0, int e0) {
+    for_each_row<ReadOnly>(c, p, bad, [&](int s0, int e0) {
         // U candidates' loads at a time, past the range's end too (xA is followed by vA in the
         // workspace)
         for (int q0 = s0; q0 < e0; q0 += U) {

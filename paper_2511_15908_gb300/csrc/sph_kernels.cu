@@ -66,7 +66,7 @@ template <int COOP, int MODE>
 __global__ void __launch_bounds__(SPH_DENSITY_THREADS, SPH_DENSITY_MINB) k_density(SimConst c)
 {
     chain_enter();
-    density_item<SPH_DENSITY_THREADS, COOP, MODE, true>(c, blockIdx.x);
+    density_item<SPH_DENSITY_THREADS, COOP, MODE, true, ReadOnly>(c, blockIdx.x);
 }
 #define SPH_SEARCH_THREADS 256
 #define SPH_SEARCH_MINB 5
@@ -74,7 +74,7 @@ template <int COOP>
 __global__ void __launch_bounds__(SPH_SEARCH_THREADS, SPH_SEARCH_MINB) k_search(SimConst c)
 {
     chain_enter();
-    search_item<SPH_SEARCH_THREADS, COOP>(c, blockIdx.x);
+    search_item<SPH_SEARCH_THREADS, COOP, ReadOnly>(c, blockIdx.x);
 }
 template <int G>
 __global__ void __launch_bounds__(kTile, SPH_LOW_LATENCY_MINB) k_density_walk(SimConst c)
@@ -91,13 +91,13 @@ __global__ void __launch_bounds__(kTile, SPH_LOW_LATENCY_MINB) k_density_lanes(S
 __global__ void __launch_bounds__(kTile) k_boundary_volume(SimConst c)
 {
     chain_enter();
-    boundary_volume_item(c, blockIdx.x);
+    boundary_volume_item<ReadOnly>(c, blockIdx.x);
 }
 template <bool VOL>
 __global__ void __launch_bounds__(kForceThreads, SPH_FORCE_MINB) k_force(SimConst c)
 {
     chain_enter();
-    force_item_v<kForceThreads, VOL>(c, blockIdx.x);
+    force_item_v<kForceThreads, VOL, ReadOnly>(c, blockIdx.x);
 }
 template <int G>
 __global__ void __launch_bounds__(kTile, SPH_FORCE_COOP_MINB) k_force_coop(SimConst c)
