@@ -147,7 +147,8 @@ struct sph_handle {
     unsigned char *pin = nullptr;
     size_t pin_bytes = 0;
     HapticSlot *slot = nullptr;          // in the same memory, behind them
-    char *pin_state = nullptr;           // and a small scene's state
+    char *pin_state = nullptr;           // and a small scene's state, up to
+    size_t pin_state_bytes = 0;          // so many bytes
 };
 
 namespace {
@@ -458,15 +459,22 @@ sph_status sph_create(const sph_params *p, const sph_capacity *cap, void *d_work
     // smoothing window's cycle log (host memory; unpinned copies if refused)
     h->pin_bytes = 64 + 16 + 48 * (size_t)c.smooth_window;
     const size_t slot_end = align256(h->pin_bytes + sizeof(HapticSlot));
-    const size_t state_bytes = 256 + 28 * (size_t)cap->max_particles;
-    const bool small = state_bytes <= kPinStateMax;
-    if (cudaHostAlloc((void **)&h->pin, slot_end + (small ? kPinStateMax : 0), cudaHostAllocDefault) != cudaSuccess) {
+    // a small scene's state behind it: 28 bytes a particle without the debug record, 44 with it
+    const size_t np = (size_t)cap->max_particles;
+    if (256 + 28 * np <= kPinStateMax) h->pin_state_bytes = std::min(256 + 44 * np, kPinStateMax);
+    cudaError_t pe = cudaHostAlloc((void **)&h->pin, slot_end + h->pin_state_bytes, cudaHostAllocDefault);
+    if (pe != cudaSuccess && h->pin_state_bytes) {
+        cudaGetLastError();
+        h->pin_state_bytes = 0;
+        pe = cudaHostAlloc((void **)&h->pin, slot_end, cudaHostAllocDefault);
+    }
+    if (pe != cudaSuccess) {
         h->pin = nullptr;
         h->pin_bytes = 0;
         cudaGetLastError();
     } else {
         h->slot = reinterpret_cast<HapticSlot *>(h->pin + h->pin_bytes);
-        if (small) h->pin_state = reinterpret_cast<char *>(h->pin + slot_end);
+        if (h->pin_state_bytes) h->pin_state = reinterpret_cast<char *>(h->pin + slot_end);
     }
     *out = h;
     return SPH_OK;
@@ -800,7 +808,7 @@ sph_status sph_get_state(sph_handle *h, float *h_x, float *h_v, float *h_rho, in
     SPH_CUDA(h, cudaMemsetAsync(d_bad, 0, 4, s));
     SPH_CUDA(h, launch_state(h->c, s, o));
     unsigned bad = 0;
-    if (h->pin_state && off <= kPinStateMax) {
+    if (h->pin_state && off <= h->pin_state_bytes) {
         // a small scene's arrays and status words in one copy through pinned memory
         SPH_CUDA(h, cudaMemcpyAsync(h->pin_state, out, off, cudaMemcpyDeviceToHost, s));
         SPH_CUDA(h, cudaStreamSynchronize(s));
