@@ -161,7 +161,7 @@ sph_status fail(sph_handle *h, sph_status s, const std::string &msg)
 
 sph_status cuda_fail(sph_handle *h, cudaError_t e, const char *where)
 {
-    return fail(h, SPH_ERR_CUDA, std::string(where) + ": " + cudaGetErrorString(e));
+    return fail(h, cuda_error(), std::string(where) + ": " + cudaGetErrorString(e));
 }
 
 #define SPH_CUDA(h, call)                                           \
@@ -453,7 +453,7 @@ sph_status sph_create(const sph_params *p, const sph_capacity *cap, void *d_work
     if (e == cudaSuccess) e = cudaStreamSynchronize(h->stream);
     if (e != cudaSuccess) {
         delete h;
-        return SPH_ERR_CUDA;
+        return cuda_error();
     }
     // pinned staging for the synchronising reads: status, then the counters and the
     // smoothing window's cycle log (host memory; unpinned copies if refused)

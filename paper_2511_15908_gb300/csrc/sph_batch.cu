@@ -272,7 +272,7 @@ sph_status bfail(sph_batch *b, sph_status s, const std::string &m)
     do {                                                                            \
         cudaError_t e_ = (call);                                                    \
         if (e_ != cudaSuccess)                                                      \
-            return bfail((b), SPH_ERR_CUDA, std::string(#call) + ": " + cudaGetErrorString(e_)); \
+            return bfail((b), cuda_error(), std::string(#call) + ": " + cudaGetErrorString(e_)); \
     } while (0)
 
 cudaError_t launch_phases(sph_batch *b, int n_substeps, int cycle_end)
@@ -367,13 +367,12 @@ sph_status capture_batch(sph_batch *b, int n_substeps, cudaGraphExec_t *out)
     cudaError_t ce = cudaStreamEndCapture(b->stream, &g);
     if (le != cudaSuccess || ce != cudaSuccess) {
         if (g) cudaGraphDestroy(g);
-        cudaGetLastError();
-        return bfail(b, SPH_ERR_CUDA, std::string("batch capture: ") +
+        return bfail(b, cuda_error(), std::string("batch capture: ") +
                                           cudaGetErrorString(le != cudaSuccess ? le : ce));
     }
     cudaError_t ie = cudaGraphInstantiate(out, g, 0);
     cudaGraphDestroy(g);
-    if (ie != cudaSuccess) return bfail(b, SPH_ERR_CUDA, std::string("batch instantiate: ") + cudaGetErrorString(ie));
+    if (ie != cudaSuccess) return bfail(b, cuda_error(), std::string("batch instantiate: ") + cudaGetErrorString(ie));
     return SPH_OK;
 }
 
@@ -482,7 +481,7 @@ sph_status sph_batch_create(sph_handle *const *scenes, int32_t n_scenes, void *d
     if (e == cudaSuccess) e = cudaStreamSynchronize(b->stream);
     if (e != cudaSuccess || b->max_bps < 1) {
         delete b;
-        return SPH_ERR_CUDA;
+        return cuda_error();
     }
     b->bps = b->max_bps;
     *out = b;

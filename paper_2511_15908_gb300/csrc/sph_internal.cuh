@@ -9,6 +9,8 @@
 #include <cstdint>
 #include <cuda_runtime.h>
 
+#include "sph.h"
+
 namespace sphgb {
 
 constexpr int kMaxBodies = 64;
@@ -143,6 +145,14 @@ inline cudaError_t launch_after(bool early, void (*kernel)(Params...), unsigned 
     cfg.attrs = attr;
     cfg.numAttrs = early ? 1 : 0;
     return cudaLaunchKernelEx(&cfg, kernel, Params(args)...);
+}
+
+// The status of a call that a CUDA error ends.  The error is taken out of the runtime's record: it
+// is this call's, and would otherwise fail the next call's check of its launches.
+inline sph_status cuda_error()
+{
+    cudaGetLastError();
+    return SPH_ERR_CUDA;
 }
 
 // Launchers (sph_kernels.cu).  All enqueue on `s` and return the launch error.

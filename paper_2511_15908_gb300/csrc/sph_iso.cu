@@ -501,10 +501,10 @@ sph_status sph_iso_field(sph_handle *h, float cube, float *d_field)
     const cudaStream_t s = scene_stream(h);
     // the hash and reorder of the current state (the next substep's own hash redoes the
     // same work from the same state), then the field from the sorted copy
-    if (c.n > 0 && launch_sort(c, s) != cudaSuccess) return SPH_ERR_CUDA;
+    if (c.n > 0 && launch_sort(c, s) != cudaSuccess) return cuda_error();
     const long long nv = (long long)g.n[0] * g.n[1] * g.n[2];
     if (c.n == 0) {
-        if (cudaMemsetAsync(d_field, 0, 4 * (size_t)nv, s) != cudaSuccess) return SPH_ERR_CUDA;
+        if (cudaMemsetAsync(d_field, 0, 4 * (size_t)nv, s) != cudaSuccess) return cuda_error();
         return SPH_OK;
     }
     if (nv <= kIsoLanesMax && c.Rc < 2.5f)         // (the cooperative walk's row table)
@@ -531,7 +531,7 @@ sph_status sph_iso_polygonize(const float *d_field, const int32_t dims[3], const
     IsoLayout L;
     if (!iso_layout(dims, L)) return SPH_ERR_ARG;
     if (!d_ws || ws_bytes < L.total || ((uintptr_t)d_ws & 255u)) return SPH_ERR_WORKSPACE;
-    if (ensure_table() != cudaSuccess) return SPH_ERR_CUDA;
+    if (ensure_table() != cudaSuccess) return cuda_error();
     const cudaStream_t s = (cudaStream_t)cuda_stream;
     char *ws = (char *)d_ws;
     uint32_t *cnt = (uint32_t *)(ws + L.cnt), *start = (uint32_t *)(ws + L.start);
@@ -554,11 +554,11 @@ sph_status sph_iso_polygonize(const float *d_field, const int32_t dims[3], const
     k_iso_scan_tiles<<<L.ntiles, kTile, 0, s>>>(c);
     k_iso_scan_apply<<<L.ntiles, kTile, 0, s>>>(c);
     if (max_tris > 0) k_iso_write<<<blocks(L.ncube), kTile, 0, s>>>(g, L.ncube, start, d_tris, max_tris);
-    if (cudaGetLastError() != cudaSuccess) return SPH_ERR_CUDA;
+    if (cudaGetLastError() != cudaSuccess) return cuda_error();
     uint32_t total = 0;
     if (cudaMemcpyAsync(&total, start + L.ncube, 4, cudaMemcpyDeviceToHost, s) != cudaSuccess)
-        return SPH_ERR_CUDA;
-    if (cudaStreamSynchronize(s) != cudaSuccess) return SPH_ERR_CUDA;
+        return cuda_error();
+    if (cudaStreamSynchronize(s) != cudaSuccess) return cuda_error();
     *h_n_tris = (int64_t)total;
     return (int64_t)total > max_tris ? SPH_ERR_CAPACITY : SPH_OK;
 }

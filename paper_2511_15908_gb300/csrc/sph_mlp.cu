@@ -920,7 +920,7 @@ sph_status mfail(sph_mlp *m, sph_status s, const std::string &msg)
     do {                                                                             \
         cudaError_t e_ = (call);                                                     \
         if (e_ != cudaSuccess)                                                       \
-            return mfail((m), SPH_ERR_CUDA, std::string(#call) + ": " + cudaGetErrorString(e_)); \
+            return mfail((m), cuda_error(), std::string(#call) + ": " + cudaGetErrorString(e_)); \
     } while (0)
 
 MlpArgs mlp_args(const sph_mlp *m, const float *d_x, int B)
@@ -1053,7 +1053,7 @@ sph_status sph_mlp_create(void *d_workspace, size_t bytes, void *cuda_stream, in
     if (e != cudaSuccess) {
         if (m->pin) cudaFreeHost(m->pin);
         delete m;
-        return SPH_ERR_CUDA;
+        return cuda_error();
     }
     *out = m;
     return SPH_OK;

@@ -119,7 +119,7 @@ extern "C" sph_status sph_cell_sort_noalloc(const sph_params *p, const float *d_
     const long long ncell = (long long)dims[0] * dims[1] * dims[2];
     if (ncell > SPH_NOALLOC_MAX_CELLS) return SPH_ERR_CAPACITY;
     uint32_t *s = nullptr;
-    if (scratch_for_current_device(&s) != cudaSuccess) return SPH_ERR_CUDA;
+    if (scratch_for_current_device(&s) != cudaSuccess) return cuda_error();
     cudaStream_t st = (cudaStream_t)cuda_stream;
     c.n = n;
     c.nf = n;
@@ -137,7 +137,7 @@ extern "C" sph_status sph_cell_sort_noalloc(const sph_params *p, const float *d_
     // the status words, the scan's tiles and the counters keep the previous call's contents: start
     // from zero.  The call is bound by its launches: one clear for two and the single-pass scan
     // for the two-pass one make five of seven (200k particles 74.5 -> 70 us a call)
-    if (cudaMemsetAsync(s, 0, 4 * (kNaCnt + (size_t)ncell + 1), st) != cudaSuccess) return SPH_ERR_CUDA;
+    if (cudaMemsetAsync(s, 0, 4 * (kNaCnt + (size_t)ncell + 1), st) != cudaSuccess) return cuda_error();
     const int nb = (n + kTile - 1) / kTile;
     if (n > 0) k_na_hash<<<nb, kTile, 0, st>>>(c);
     k_na_scan<<<c.n_scan_tiles, kTile, 0, st>>>(c);
