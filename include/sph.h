@@ -148,7 +148,8 @@ typedef struct {
 } sph_capacity;
 
 /* Bytes of device workspace a scene with these parameters and capacities needs
- * (0 if the arguments are invalid).  The grid size follows from domain and cell; with
+ * (0 if the arguments are invalid).  256 bytes and 44 per particle of it are the state in id
+ * order that sph_get_state copies from.  The grid size follows from domain and cell; with
  * SPH_FLAG_LOW_LATENCY the force pass's diagnostic rows take up to 4 times their usual
  * 512 bytes per 1,024 particles (so the flag is part of the parameters the size is
  * computed for). */

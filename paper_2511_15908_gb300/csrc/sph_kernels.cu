@@ -5,8 +5,9 @@
 // Block shape and resident blocks per SM each pass is built for (its register budget).
 // Measured (us, search + sums): search in 256-thread blocks at 5 blocks per SM, 48 registers
 // (6 blocks, 40 registers: coupled 1.16 M 437 against 409; 4: the same); density sums at 4
-// blocks, 64 registers, with the next quad's neighbours in flight (5 blocks spill: 476 against
-// 414; 3 blocks: 422); force in 128-thread blocks, 6 per SM, 80 registers: the pass waits for its
+// blocks, 64 registers, with the next quad's neighbours in flight (their instances spill 12 to
+// 68 bytes; 5 blocks spill more: 476 against 414; 3 blocks: 422); force in 128-thread blocks, 6
+// per SM, 80 registers (spilling 16 bytes, the volume variant 100): the pass waits for its
 // gathers (4 bytes of list and 40 of state a partner), which more warps hide better than loads
 // issued ahead (coupled 1.16 M: 224; 5 blocks of 96 registers 233, the next two partners
 // fetched ahead at 5 / 4 blocks 297 / 264, 7 blocks 227), and blocks of 256 leave a longer last
@@ -196,8 +197,9 @@ __global__ void k_sorted_keys(SimConst c, uint32_t *keys, int *ids)
 
 // The state in id order for the caller (one thread per slot; the scattered stores stay in L2).
 // A host loop over the slots, after copies of 40 bytes a particle into buffers of its own, took
-// most of a read: 32 substeps of the 365k stirring tank and a read 11.2 ms, now 9.4; 100 of the
-// 1.16 M coupled scene 72.3 ms, now 66.0.
+// most of a read.  With this kernel and the pages of the caller's arrays populated ahead of the
+// copies (sph_get_state), together: 32 substeps of the 365k stirring tank and a read 11.2 ms, now
+// 9.4; 100 of the 1.16 M coupled scene 72.3 ms, now 66.0.
 __global__ void __launch_bounds__(kTile) k_state(SimConst c, StateOut o)
 {
     const int p = blockIdx.x * kTile + threadIdx.x;
@@ -230,10 +232,15 @@ __global__ void __launch_bounds__(kTile) k_state(SimConst c, StateOut o)
 //     stirring tank 127 against 137; 85k of the coupled scene 113 against 78;
 //   rigid particles, 4 lanes, up to 900,000 particles: 307k of the coupled scene 103 against
 //     159, the 365k stirring tank (18.7k of them rigid) 156 against 184; 2 lanes 161 / 160,
-//     8 lanes 108 / 166.  The 1.16 M coupled scene lasts longer than its rigid chains (389 with
-//     4 lanes against 385).  With more than an eighth of all particles rigid their number hides
-//     the chains, and the lanes' overhead would show;
+//     8 lanes 108 / 166;
 //   nobody else.
+// Around the two lines (whole substep, us, 4 lanes / one thread).  Coupled scene from its fill,
+// 30k / 7k rigid particles: 0.5 M particles 359 / 387 and 274 / 333, 0.8 M 487 / 495 and 401 /
+// 440, 0.98 M 544 / 551 and 465 / 488, 1.15 M 619 / 621 and 544 / 559; from its stirred state the
+// 1.16 M scene's search and sums took 389 / 385.  So 900,000 lies where the gain runs out for a
+// large body, early for a small one.  Share of rigid particles: 12 % 155 / 225 (130k), 16 % 349 /
+// 390, 24 % 440 / 464 and 224 / 259, 38 % 646 / 687, 55 % 1090 / 1058 (656k): the lanes pay well
+// beyond an eighth, which is on the safe side of where they cross.
 constexpr int kCoopAllMax = 60000, kCoopRigidMax = 900000;
 int walk_coop(const SimConst &c)
 {

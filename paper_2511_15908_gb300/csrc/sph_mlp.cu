@@ -536,7 +536,7 @@ __global__ void __launch_bounds__(128, 1)
 // and every rounding is that of the single GEMMs.  What the epilogues take (16 k GELUs a stage
 // and CTA, ~2 us) bounds the kernel; a batch of 1024 has eight CTAs.
 // Training also writes the column-major BF16 copies ([feature][batch]) that the weight
-// gradients contract over the batch, keeps the pre-activations Z for the backward stages
+// gradients contract over the batch, keeps GELU's derivatives for the backward stages
 // ([tile][column][row], each thread reads what it wrote), and writes the partials of the loss
 // (FP64, per 16 rows) and of the bias gradients (per tile; db4 per 16 rows), each in a fixed
 // order.

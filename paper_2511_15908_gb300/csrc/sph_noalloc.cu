@@ -135,8 +135,9 @@ extern "C" sph_status sph_cell_sort_noalloc(const sph_params *p, const float *d_
     c.perm = c.rank + SPH_NOALLOC_MAX_PARTICLES;
     c.cell_start = d_cell_start;
     // the status words, the scan's tiles and the counters keep the previous call's contents: start
-    // from zero.  The call is bound by its launches: one clear for two and the single-pass scan
-    // for the two-pass one make five of seven (200k particles 74.5 -> 70 us a call)
+    // from zero.  The call is bound by its launches and the host's side of them: one clear for two
+    // and the single-pass scan for the two-pass one make five of seven (200k particles 74.5 -> 70
+    // us a call in one pair of runs, within what calls differ by in others)
     if (cudaMemsetAsync(s, 0, 4 * (kNaCnt + (size_t)ncell + 1), st) != cudaSuccess) return cuda_error();
     const int nb = (n + kTile - 1) / kTile;
     if (n > 0) k_na_hash<<<nb, kTile, 0, st>>>(c);
