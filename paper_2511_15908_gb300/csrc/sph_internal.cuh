@@ -25,7 +25,7 @@ constexpr int kMaxCell = 512;       // particles per cell for the deterministic 
 constexpr int kLowLatencyForceG = SPH_LOW_LATENCY_FORCE_G;
 constexpr int kForceThreads = 128;  // particles per block (and diagnostic row) of the force pass
 // Scenes of at most kForceOrderedMax particles whose walk cooperates throughout (SimConst::coop
-// 2): the force pass takes kForceOrderedG lanes per particle (dam break, 12k particles: 20.5 us
+// 3): the force pass takes kForceOrderedG lanes per particle (dam break, 12k particles: 20.5 us
 // with one thread each, 12.3 with the lanes; from 29k on they gain nothing: 20.5 / 22.5).
 constexpr int kForceOrderedG = 8, kForceOrderedMax = 20000;
 constexpr int kScanTile = 2048;     // cells per scan block (256 threads x 8)
@@ -57,8 +57,8 @@ struct DevBody {
 struct __align__(16) SimConst {
     int n, nf, nb, n_body_particles;
     int n_rigid;               // particles of rigid bodies
-    int coop;                  // who walks with cooperating lanes (walk_role): 0 nobody, 1 rigid
-                               // particles, 2 every particle
+    int coop;                  // who walks with cooperating lanes (walk_role): 0 nobody, 1 and 2
+                               // rigid particles, 3 every particle
     int nx, ny, nz, ncell;
     float o[3], inv_cell;
     float R2, h, inv_h;

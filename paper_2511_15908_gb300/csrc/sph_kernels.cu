@@ -225,33 +225,42 @@ __global__ void __launch_bounds__(kTile) k_state(SimConst c, StateOut o)
 
 // ----------------------------------------------------------------------- launchers
 
-// Who walks with cooperating lanes (same results either way; us of search + density sum):
-//   every particle, 16 lanes, in scenes of up to 60,000: dam break (12k particles) 31 (8 lanes
-//     41, 32 lanes 38) against 112 with one thread each, where a cube particle's ~226
-//     neighbours form one chain; 45k particles of the coupled scene 71.6 against 75; a 58k
-//     stirring tank 127 against 137; 85k of the coupled scene 113 against 78;
-//   rigid particles, 4 lanes, up to 900,000 particles: 307k of the coupled scene 103 against
-//     159, the 365k stirring tank (18.7k of them rigid) 156 against 184; 2 lanes 161 / 160,
-//     8 lanes 108 / 166;
-//   nobody else.
-// Around the two lines (whole substep, us, 4 lanes / one thread).  Coupled scene from its fill,
+// Who walks with cooperating lanes (same results either way; us).  Lanes shorten the chain of a
+// particle alone in its lane, a rigid one's ~226 neighbours above all, and cost work: a scene alone
+// gains while it leaves the GPU room, scenes stepped side by side on their own streams pay.
+//   3: every particle, 16 lanes, in scenes of up to 30,000.  Search and density sum of the dam break
+//     (12k particles) 31 (8 lanes 41, 32 lanes 38) against 112 with one thread each.
+//   2: rigid particles, 8 lanes, up to 60,000.  Whole substep with 3 / 2, alone and per substep of
+//     8 scenes side by side: 22k coupled 92 / 103 and 321 / 206, 27k stirring 95 / 101 and 384 /
+//     227, 30k coupled 99 / 103 and 398 / 216, 33k stirring 104 / 97 and 463 / 256; alone 42k coupled
+//     108 / 102, 40k, 52k and 58k stirring 109 / 99, 128 / 114 and 135 / 117.  One thread each: 30k
+//     coupled 214 and 301, 33k stirring 180 and 285 (that walk from before the search and the sums
+//     were split).  Below 30,000 a scene alone counts; 64 scenes or more of a few thousand particles
+//     take longer side by side than one thread each did (256 of 6.5k to 17k: 5.2 ms for 2.7 a
+//     substep), and 2.2 in a batch, which walks with one thread each.
+//   1: rigid particles, 4 lanes, up to 900,000: 307k of the coupled scene 103 against 159 (search and
+//     sum), the 365k stirring tank (18.7k of them rigid) 156 against 184; 2 lanes 161 / 160, 8 lanes
+//     108 / 166.
+//   0: nobody else.
+// Around 1's two lines (whole substep, 4 lanes / one thread).  Coupled scene from its fill,
 // 30k / 7k rigid particles: 0.5 M particles 359 / 387 and 274 / 333, 0.8 M 487 / 495 and 401 /
 // 440, 0.98 M 544 / 551 and 465 / 488, 1.15 M 619 / 621 and 544 / 559; from its stirred state the
 // 1.16 M scene's search and sums took 389 / 385.  So 900,000 lies where the gain runs out for a
 // large body, early for a small one.  Share of rigid particles: 12 % 155 / 225 (130k), 16 % 349 /
 // 390, 24 % 440 / 464 and 224 / 259, 38 % 646 / 687, 55 % 1090 / 1058 (656k): the lanes pay well
 // beyond an eighth, which is on the safe side of where they cross.
-constexpr int kCoopAllMax = 60000, kCoopRigidMax = 900000;
+constexpr int kCoopAllMax = 30000, kCoopEightMax = 60000, kCoopRigidMax = 900000;
 int walk_coop(const SimConst &c)
 {
     if (c.Rc >= 2.5f) return 0;                 // the cooperative search's row table
-    return c.n <= kCoopAllMax ? 2 : c.n <= kCoopRigidMax && c.n_rigid <= c.n / 8 ? 1 : 0;
+    if (c.n <= kCoopEightMax) return c.n <= kCoopAllMax ? 3 : 2;
+    return c.n <= kCoopRigidMax && c.n_rigid <= c.n / 8 ? 1 : 0;
 }
 
 static bool force_low_latency(const SimConst &c) { return (c.flags & FLAG_LOW_LATENCY) && !(c.flags & FLAG_VOLUME); }
 static bool force_ordered(const SimConst &c)
 {
-    return c.coop == 2 && c.n <= kForceOrderedMax && !(c.flags & (FLAG_VOLUME | FLAG_LOW_LATENCY));
+    return c.coop == 3 && c.n <= kForceOrderedMax && !(c.flags & (FLAG_VOLUME | FLAG_LOW_LATENCY));
 }
 int force_blocks(const SimConst &c)
 {
@@ -303,17 +312,20 @@ cudaError_t launch_substep(const SimConst &c, cudaStream_t s, cudaEvent_t *ev, b
     // boundary weights between them.  The low-latency pass's walk has rows for Rc < 2.5 (cells >= h
     // give Rc ~ 2)
     const bool lanes = force_low_latency(c) && c.Rc < 2.5f, walk = lanes && c.n <= kLowLatency32Max;
-    const auto search = c.coop == 0 ? k_search<0> : c.coop == 1 ? k_search<1> : k_search<2>;
+    const auto search = c.coop == 0 ? k_search<0> : c.coop == 1 ? k_search<1> : c.coop == 2 ? k_search<2> : k_search<3>;
     if (!walk) go(search, search_tiles(c, SPH_SEARCH_THREADS), SPH_SEARCH_THREADS, false);
     if (walk) {
-        go(k_density_walk<32>, (unsigned)tiles_of<32>(c.n, kTile), kTile, false);
+        go(k_density_walk<32>, (unsigned)tiles_of(c.n, 32, kTile), kTile, false);
     } else if (lanes) {
-        go(k_density_lanes<16>, (unsigned)tiles_of<16>(c.n, kTile), kTile, false);
+        go(k_density_lanes<16>, (unsigned)tiles_of(c.n, 16, kTile), kTile, false);
     } else {
         const bool vol = (c.flags & FLAG_VOLUME) != 0;
         if (vol && c.n > c.nf) go(k_boundary_volume, blocks_for(c.n - c.nf, kTile), kTile, false);
-        const auto density = vol ? (c.coop == 0 ? k_density<0, DENSITY_VOLUME> : c.coop == 1 ? k_density<1, DENSITY_VOLUME> : k_density<2, DENSITY_VOLUME>)
-                                 : (c.coop == 0 ? k_density<0, DENSITY_MASS> : c.coop == 1 ? k_density<1, DENSITY_MASS> : k_density<2, DENSITY_MASS>);
+        const auto of_mass = c.coop == 0 ? k_density<0, DENSITY_MASS> : c.coop == 1 ? k_density<1, DENSITY_MASS>
+                             : c.coop == 2 ? k_density<2, DENSITY_MASS> : k_density<3, DENSITY_MASS>;
+        const auto of_volume = c.coop == 0 ? k_density<0, DENSITY_VOLUME> : c.coop == 1 ? k_density<1, DENSITY_VOLUME>
+                               : c.coop == 2 ? k_density<2, DENSITY_VOLUME> : k_density<3, DENSITY_VOLUME>;
+        const auto density = vol ? of_volume : of_mass;
         go(density, density_tiles(c, SPH_DENSITY_THREADS), SPH_DENSITY_THREADS, false);
     }
     mark();
