@@ -135,7 +135,7 @@ __global__ void __launch_bounds__(kTile, SPH_BATCH_MINB) k_batch(BatchConst b, i
                     }
                     __syncthreads();
                     const SimConst &c = s_c;
-                    const int blk = t.blk + (t.rest ? rigid_tiles(c, kTile) : 0);
+                    const int blk = t.blk + (t.rest ? tiles_of(c.n_rigid, rigid_lanes(0), kTile) : 0);
                     switch (ph) {
                     case P_HASH: hash_item(c, blk); break;
                     case P_SCAN: scan_lookback_item(c); break;
@@ -183,7 +183,7 @@ __global__ void __launch_bounds__(kTile, batch_phase_minb<PH>()) k_batch_phase(B
     }
     __syncthreads();
     const SimConst &c = s_c;
-    const int blk = t.blk + (t.rest ? rigid_tiles(c, kTile) : 0);
+    const int blk = t.blk + (t.rest ? tiles_of(c.n_rigid, rigid_lanes(0), kTile) : 0);
     switch (PH) {
     case P_HASH: hash_item(c, blk); break;
     case P_SCAN: scan_lookback_item(c); break;
